@@ -173,7 +173,8 @@ hd_status_t sfa_bwd(const void* q, const void* k, const void* v, const void* o, 
  *   sfa_bwd_prep     : delta = rowsum(dO * O) and lse * log2(e) into the workspace
  *                      (fp32, stream-major), and zero its fp32 dQ accumulator.
  *   sfa_bwd_main     : recompute P on visible pairs, add every dQ contribution
- *                      into the accumulator and write dk, dv (overwritten).
+ *                      into the accumulator (at Dh = 256: store the finished sums
+ *                      there) and write dk, dv (overwritten).
  *   sfa_bwd_finalize : dq = bf16(scale * accumulator).
  * A later phase reads what the earlier one left in the workspace.
  * sfa_bwd_prep is itself the two halves below, for a caller that overlaps them:

@@ -63,7 +63,9 @@ __host__ __device__ inline int row_terms_pitch(int Lv) { return (Lv + kRowTermAl
 // traffic cost more than the better balance gained: 3 % slower.)  Chunk hc writes its dK / dV partial sums (fp32,
 // dK already scaled) to its own slice of a workspace [chunks][2][B][q_ns][Lv][Hkv][Dh]
 // (dV, then dK), and a finalize pass adds the slices in chunk order: the same result,
-// bit for bit, on every run.
+// bit for bit, on every run.  This rule sizes the workspace at every head dim; the
+// head-dim-256 kernel has another grid and chooses its own chunk count (head_chunks in
+// sfa_bwd_tc256.cu) within that space.
 constexpr int kSmCount = 152;
 __host__ __device__ inline int bwd_head_chunks(const SfaGeom& g, int Dh) {
   const long long ctas = (long long)((g.Lv + 127) / 128) * (Dh == 256 ? 2 : 1) * g.Hkv * g.q_ns * g.B;

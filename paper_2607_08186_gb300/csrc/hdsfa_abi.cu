@@ -36,8 +36,8 @@ cudaError_t launch_sfa_bwd_main_tc(const void* q, const void* k, const void* v, 
                                    void* dv, const float* lse2_ws, const float* delta_ws, float* dq_ws,
                                    float* dkv_ws, const SfaGeom& g, int Dh, float scale, int32_t* status,
                                    cudaStream_t st);
-cudaError_t launch_sfa_bwd_main_tc256(const void* q, const void* k, const void* v, const void* dout, void* dk,
-                                      void* dv, const float* lse2_ws, const float* delta_ws, float* dq_ws,
+cudaError_t launch_sfa_bwd_main_tc256(const void* q, const void* k, const void* v, const void* dout, void* dq_out,
+                                      void* dk, void* dv, const float* lse2_ws, const float* delta_ws, float* dq_ws,
                                       float* dkv_ws, const SfaGeom& g, float scale, int32_t* status,
                                       cudaStream_t st);
 cudaError_t launch_sfa_bwd_finalize(void* dq, const float* dq_ws, const SfaGeom& g, int Dh,
@@ -303,11 +303,10 @@ hd_status_t sfa_bwd_main(const void* q, const void* k, const void* v, const void
   BwdWs ws;
   if ((st = split_ws(g, Dh, workspace, workspace_bytes, &ws)) != HD_OK) return st;
   const float scale = resolve_scale(softmax_scale, Dh);
-  // tcgen05 kernels at every head dim (at 256 as two CTAs per key tile, one per half
-  // of the dK / dV / dQ columns)
+  // tcgen05 kernels at every head dim (at 256 the accumulator is stored, not added to)
   if (Dh == 256)
-    return cuda_status(hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g,
-                                                        scale, dev_status, stream));
+    return cuda_status(hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, nullptr, dk, dv, ws.lse2, ws.delta, ws.dq,
+                                                        ws.dkv, g, scale, dev_status, stream));
   return cuda_status(hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, Dh,
                                                    scale, dev_status, stream));
 }
@@ -340,6 +339,14 @@ hd_status_t sfa_bwd(const void* q, const void* k, const void* v, const void* o, 
   if (st != HD_OK) return st;
   BwdWs ws;
   if ((st = split_ws(g, Dh, workspace, workspace_bytes, &ws)) != HD_OK) return st;
+  if (Dh == 256) {  // dQ leaves the main pass as bf16: no accumulator to clear or convert
+    const float scale = resolve_scale(softmax_scale, Dh);
+    cudaError_t e = hdsfa::launch_sfa_bwd_prep(o, dout, lse, ws.lse2, ws.delta, ws.dq, query_geom(g), Dh, stream, false);
+    if (e == cudaSuccess)
+      e = hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, scale,
+                                           dev_status, stream);
+    return cuda_status(e);
+  }
   st = sfa_bwd_prep(o, dout, lse, B, L, n, Hq, Hkv, Dh, mode, workspace, workspace_bytes, stream);
   if (st != HD_OK) return st;
   st = sfa_bwd_main(q, k, v, dout, dk, dv, B, L, n, Hq, Hkv, Dh, softmax_scale, mode, window, workspace,
@@ -434,7 +441,7 @@ hd_status_t sfa_bwd_final(const void* q, const void* k, const void* v, const voi
   if ((st = split_ws(g, Dh, workspace, workspace_bytes, &ws)) != HD_OK) return st;
   const float scale = resolve_scale(softmax_scale, Dh);
   const SfaGeom gq = query_geom(g);
-  cudaError_t e = hdsfa::launch_sfa_bwd_prep(o, dout, lse, ws.lse2, ws.delta, ws.dq, gq, Dh, stream);
+  cudaError_t e = hdsfa::launch_sfa_bwd_prep(o, dout, lse, ws.lse2, ws.delta, ws.dq, gq, Dh, stream, Dh != 256);
   if (e == cudaSuccess && mode == SFA_WITHIN) {
     // only stream n-1's keys are seen by the final-stream queries: the other rows are zero
     const size_t bytes = (size_t)B * n * L * Hkv * Dh * 2;
@@ -443,13 +450,13 @@ hd_status_t sfa_bwd_final(const void* q, const void* k, const void* v, const voi
   }
   if (e == cudaSuccess) {
     if (Dh == 256)
-      e = hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, scale, dev_status,
-                                           stream);
+      e = hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, scale,
+                                           dev_status, stream);
     else
       e = hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, Dh, scale, dev_status,
                                         stream);
   }
-  if (e == cudaSuccess) e = hdsfa::launch_sfa_bwd_finalize(dq, ws.dq, gq, Dh, scale, stream);
+  if (e == cudaSuccess && Dh != 256) e = hdsfa::launch_sfa_bwd_finalize(dq, ws.dq, gq, Dh, scale, stream);
   return cuda_status(e);
 }
 

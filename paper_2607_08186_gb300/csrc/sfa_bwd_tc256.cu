@@ -2,45 +2,60 @@
 // head dim 256 (the 80B configuration's heads, Table 6).
 //
 // The gradient is the one of the head-dim-128 kernel (derivative of the forward of
-// Eq. 4 / Fig. 2, which the paper trains through, Sec. 3.1); the tile plan differs
-// because at head dim 256 a 128-row key tile's dK and dV alone would fill the 512
-// TMEM columns, and its K and V tiles take 128 KB of shared memory:
-//   * Two CTAs per 128-row key tile, one per half c of the head dim: each computes
-//     S^T and dP^T over the full head dim (the two CTAs of a key tile compute them
-//     both, 1.4x the algorithmic FLOPs) and accumulates only its half of dK, dV and
-//     dQ.
-//   * 64-row query tiles, so K and V stay resident (64 KB each) beside the query
-//     tile: Q as its other head-dim half (single buffer: read only by S^T, released
-//     after S^T's first eight k-steps) and its own half (double buffer: read by S^T
-//     and, at the end of the tile, by dK_c), dO single-buffered (32 KB), dS^T (16 KB).
-//   * TMEM: two region pairs, one per tile parity p, each an S'^T region RS(p) and a
-//     dP'^T region RD(p) of 64 columns (columns 0..255), dV_c at 256, dK_c at 384.
-//     While the softmax works on tile t in pair p, S^T and dP^T of tile t+1 fill
-//     pair p^1.
-//   GEMMs per 64-row query tile (M = 128 throughout):
-//     S'^T  = K Q^T  - lse2/c2 (-inf where masked)  SS, N = 64, 16 k-steps over d
-//     dP'^T = V dO^T - delta                        SS, N = 64, 16 k-steps
-//     dV_c += P^T dO[:, c]                          TS, N = 128, 4 k-steps over queries
-//     dK_c += dS^T Q[:, c]                          TS, N = 128, 4 k-steps
-//     dQ_c^T = K[:, c]^T dS^T                       SS, N = 64, 8 k-steps over keys
-//   (dQ transposed: a 64-row dQ tile would need an M = 64 MMA; its TMEM lane is a
-//   head-dim column.)  dQ_c^T(t) lands in RS(p) once P^T(t) is consumed, leaves TMEM
-//   through the dQ warps, staged in shared memory over the dS^T buffer (free once
-//   dQ_c^T has read it) and added into the fp32 accumulator by TMA tensor reduce-add.
-// Small grids (fewer CTAs than SMs: short or final-stream problems with two K/V heads)
-// also split the group's query heads into chunks, one CTA each; each chunk
-// writes its fp32 dK / dV partial sums to a workspace slice of its own, which
-// dkv_finalize_kernel adds in chunk order (bwd_head_chunks in common.cuh).
-// Roles (512 threads, at most 128 registers each): warp 0 TMA producer (+ TMEM owner);
-// three MMA issuers on different warps, each waiting only for its own operands:
-// warp 1 (one lane) dV_c and dK_c per 16-query quarter, warp 14 (whole warp, an
-// elected lane issues) S and dP, warp 15 (likewise) dQ; warps 2..5 softmax (TMEM lane
-// = key row, 64 query columns in four 16-column chunks per phase); warps 6..13
-// pre-fills and dQ: warp (6 + 4h + q) pre-fills query columns [32h, 32h + 32) of TMEM
-// lane quadrant q and reads dQ_c^T's head-dim rows [32q, 32q + 32) for queries
-// [32h, 32h + 32).  Barriers signalled once per tile are kept per tile parity, so
-// one never completes twice before its waiter has seen the first completion.
-// Every mbarrier wait is bounded.
+// Eq. 4 / Fig. 2, which the paper trains through, Sec. 3.1); the plan differs because
+// at head dim 256 dK and dV of one 128-row key tile alone would fill the 512 TMEM
+// columns.  Each gradient therefore has its own work items, in one launch:
+//   DV  key rows stationary:   S^T = K Q^T, P^T;                  dV += P^T dO
+//   DK  key rows stationary:   S^T = K Q^T, dP^T = V dO^T, dS^T;  dK += dS^T Q
+//   DQ  query rows stationary: S = Q K^T,   dP = dO V^T,   dS;    dQ += dS K
+// S is computed three times and dP twice (8 GEMMs for 5 algorithmic ones), but every
+// gradient is accumulated in TMEM over its whole loop and leaves once: no fp32 dQ
+// accumulator in HBM, no reduce-adds, no shared-memory copy of dS.
+//
+// What bounds it: the tensor pipe.  A 128 x 128 x 16 MMA with both operands in shared
+// memory reads 8 KB there in its 64 cycles, all of the SM's 128 B per clock, before any
+// TMA write; so a pair of CTAs works on 256 stationary rows (cta_group::2, M = 256):
+// each CTA holds its own 128 rows of A but only half of every B tile, 6 KB per 64
+// cycles, and the pair loads each streamed tile once.  Per 128 streamed rows a CTA's
+// shared memory moves 320 KB (2500 cycles) under 3072 cycles of MMA (DV: 192 KB under
+// 2048).
+// Measured, 80B-class WITHIN layer (B=1, L=4096, n=4, 24 over 2 heads; fwd + bwd): 4.16 ms
+// with the fused form before (one CTA per key tile and head-dim half, S and dP computed
+// by both halves, dQ added into an fp32 accumulator by TMA reduce: 3.34 ms of it, about
+// 4900 cycles per 128 x 64 tile against 3250 of its shared-memory traffic), 2.85 ms with
+// this one (2.1 ms); final-stream CROSS layer of the same heads 3.84 -> 2.49 ms.  A step
+// takes about 2500 (DV) and 3500 to 4200 (DQ, DK) cycles: what is left over the MMAs is
+// the chain dP complete -> dS -> out issued (about 1800 cycles through two cross-CTA
+// signals, 1024 of them under S(t+1)).
+//
+// A pair's work item (cluster of two CTAs, 320 threads each, one CTA per SM):
+//   A1, A2   stationary operands, 128 rows x 256 per CTA (DV: A1 only), loaded once
+//   ring     streamed operands in 16 KB pieces of 64 rows x 128 columns, in the order
+//            the issuer consumes them.  As B of S and dP (K-major, N = 128) CTA r holds
+//            streamed rows [64r, 64r+64), two pieces over the head dim; as B of the
+//            output GEMM (MN-major, N = 256) it holds head-dim columns [128r, 128r+128),
+//            two pieces over the rows.
+//   TMEM     output in columns 256..511; DQ, DK: S in 0..127, dP in 128..255 (dS packed
+//            bf16 over it, each 64-column half at the start of its own columns); DV: S
+//            double-buffered in 0..255 (P^T packed over its buffer likewise).
+//   issue    DQ, DK: S(0) dP(0) S(1), then per step t: out(t) dP(t+1) S(t+2).  The
+//            softmax takes S(t+1) into registers while out(t) and dP(t+1) run and dP(t+1)
+//            while S(t+2) runs, so the pipe does not wait for it.
+//            DV: S(0), then per step t: S(t+1) out(t).
+// Roles per CTA: warp 0 TMA producer (+ TMEM owner); warp 1 MMA issuer (the pair's first
+// CTA only: the whole warp runs the loop, one elected lane issues); warps 2..9 softmax,
+// two threads per stationary row (TMEM lane), each half of the streamed columns.  A full barrier lives in the first CTA
+// and counts both CTAs' bytes; commits are multicast to both CTAs.
+// DQ's two 128-row tiles are the same rows of two heads of one K/V group where the group
+// has an even number of heads (same key range), else consecutive tiles of one head; DK's
+// and DV's are consecutive key tiles.
+// Order of the items: DK (three GEMMs per step) and DV, key tiles with the most query
+// tiles first, then DQ, whose items are short and fill the tail.  When there are too few
+// key items to balance the SMs, each takes only a chunk of the group's query heads
+// (head_chunks below), writing fp32 partial sums that dkv_finalize_kernel adds in chunk
+// order: the same bits on every run, as for every output of this kernel.
+// Every mbarrier wait is bounded; copies still in flight when a wait gives up were issued
+// a whole timeout (about a second) earlier.
 #include "tc_common.cuh"
 
 namespace hdsfa {
@@ -48,48 +63,150 @@ namespace hdsfa {
 typedef __nv_bfloat16 bf16;
 
 namespace tcbwd256 {
-constexpr int BK = 128, BQ = 64, DH = 256, DHH = 128, NTHREADS = 512;
-constexpr int kWarpSP = 14, kWarpDQ = 15;  // issuers of S / dP and of dQ
-constexpr uint32_t COL_DV = 256, COL_DK = 384;
-HD_DEVINLINE uint32_t col_s(int p) { return 128u * p; }       // RS(p)
-HD_DEVINLINE uint32_t col_d(int p) { return 128u * p + 64u; }  // RD(p)
+constexpr int BM = 128, BN = 128, DH = 256, NTHREADS = 320;
+constexpr int PR = 64, PC = 128;               // a ring piece: rows x columns
+constexpr int HB = 64;                         // streamed columns of one softmax thread
+constexpr int NSLOT = 6, NSLOT_DV = 10;        // DV streams through A2's space as well
+constexpr uint32_t COL_OUT = 256, COL_D = 128;  // output; dP (DV: the second S buffer)
+enum Kind { kDK = 0, kDV = 1, kDQ = 2 };
 
 struct Smem {
-  bf16 k[BK * DH];        // four swizzle blocks of [128 key rows][64]
-  bf16 v[BK * DH];
-  bf16 qo[BQ * DHH];      // the query tile's other head-dim half: two blocks of [64][64]
-  bf16 qc[2][BQ * DHH];   // its own half, double-buffered
-  bf16 dO[BQ * DH];       // four blocks of [64][64]
-  bf16 ds[BK * BQ];       // dS^T [128 key rows][64 queries], one block; then dQ staging
-  float nlse2[2][BQ];     // -lse*log2(e) of the query tile in qc[i]
-  float ndelta[2][BQ];    // -delta of the query tile in qc[i]
-  uint64_t kv_full, q_full[2], qo_empty, qc_empty[2], do_full, do_empty, pa_part[4], pb_part[4], ds_free,
-      kv_done, drain;
-  uint64_t s_full[2], dp_full[2], dq_full[2], s_init[2], dp_init[2], dv_done[2], dk_done[2];  // per parity
+  bf16 a1[BM * DH];           // four [128 rows][64] swizzle blocks
+  bf16 a2[BM * DH];           // DV: ring slots 0..3
+  bf16 ring[NSLOT][PR * PC];  // piece: two [64 rows][64] swizzle blocks
+  float nlse2[2][BN];         // DK, DV: -lse*log2(e) of the streamed query tile, by step parity (loaded by bulk copy)
+  float ndelta[2][BN];        // DK: -delta of it
+  uint64_t full[NSLOT_DV], empty[NSLOT_DV], a1_full, a2_full;
+  uint64_t s_full[2], s_empty, dp_full, p_full[2], out_done, term_full[2], term_empty[2];
   uint32_t tmem_base;
   int abort;
 };
-
-constexpr int kSmemBytes = 232448;
-static_assert(sizeof(Smem) + 1024 <= kSmemBytes, "head-dim-256 backward shared memory exceeds 227 KB");
+// The layout needs 1024-byte alignment; the kernel checks the actual pad on entry.
+constexpr int kSmemBytes = sizeof(Smem) + 1024 < 232448 ? (int)sizeof(Smem) + 1024 : 232448;
+static_assert(sizeof(Smem) <= 232448, "head-dim-256 backward shared memory exceeds 227 KB");
 
 struct Params {
-  CUtensorMap tm_q, tm_do, tm_k, tm_v, tm_dq;
-  const float* lse2;   // [B][Hq][ns][Lvp]
-  const float* delta;  // [B][Hq][ns][Lvp]
+  CUtensorMap tm_q, tm_do, tm_k, tm_v;  // boxes of 64 rows x 64 columns
+  const float* lse2;   // -lse*log2(e), [B][Hq][ns][Lvp]
+  const float* delta;  // -delta, the same layout
+  bf16* dq;            // dQ (scaled), or null: dq_acc
+  float* dq_acc;       // unscaled fp32 dQ, when dq is null
   bf16* dk;
   bf16* dv;
   float* dkv;   // head chunks > 1: fp32 partial sums [chunks][2][B][q_ns][Lv][Hkv][DH] (dV, dK)
-  int hchunks;  // query-head chunks per K/V head (bwd_head_chunks)
+  int hchunks;  // query-head chunks per K/V head
+  int nkv;      // DK items (= DV items); DQ items follow
+  int head_pairs;
   SfaGeom g;
   float scale, scale_log2;
   int32_t* status;
 };
 
-// WIN: a windowed (LOCAL) problem, whose pre-fill masks only tiles that reach the
-// window edge; the other modes keep a separate instantiation.
-template <bool WIN>
-__global__ void __launch_bounds__(NTHREADS, 1) bwd256_kernel(const __grid_constant__ Params P) {
+// Arrive on the barrier at the same place in the pair's first CTA.
+HD_DEVINLINE uint32_t lead_addr(const void* p) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, 0;\n" : "=r"(r) : "r"(smem_u32(p)));
+  return r;
+}
+HD_DEVINLINE void arrive_lead(uint32_t lead_bar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];\n" ::"r"(lead_bar) : "memory");
+}
+// Load into this CTA's shared memory, counted on the first CTA's barrier.
+HD_DEVINLINE void tma_load_pair(void* dst, const CUtensorMap* m, uint32_t lead_bar, int c0, int c1, int c2, int c3,
+                                int c4) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5, %6, %7}], [%2];\n" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(lead_bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+      : "memory");
+}
+HD_DEVINLINE void mma2_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
+  asm volatile(
+      "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(accum));
+}
+HD_DEVINLINE void mma2_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
+  asm volatile(
+      "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+      "r"(a), "l"(b), "r"(idesc), "r"(accum));
+}
+// Arrive on `bar` of both CTAs once every MMA issued so far has completed.
+HD_DEVINLINE void commit2(uint64_t* bar) {
+  asm volatile(
+      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}\n" ::
+          "r"(smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+HD_DEVINLINE void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;\n" ::: "memory");
+}
+
+// One work item: its kind, stationary rows and the streamed steps.
+struct Item {
+  int kind;
+  int b, s, sk, kvh, hc;
+  int row0, head;    // this CTA's first stationary row; its query head (DQ)
+  int h_base, grp;   // DK, DV: first query head and number of heads of the chunk
+  int lo, nst;       // first streamed tile and tiles per head
+  int T;             // steps: DQ nst, DK / DV grp * nst
+};
+
+HD_DEVINLINE Item make_item(const Params& P, int idx, int rank) {
+  const SfaGeom& G = P.g;
+  Item it;
+  it.kind = idx < P.nkv ? kDK : idx < 2 * P.nkv ? kDV : kDQ;
+  it.hc = 0;
+  if (it.kind != kDQ) {
+    if (it.kind == kDV) idx -= P.nkv;
+    const int HC = P.hchunks, per_tile = HC * G.Hkv * G.q_ns * G.B;
+    const int j = idx / per_tile, rem = idx % per_tile;  // key-tile pair slowest
+    it.hc = rem % HC;
+    const int hsb = rem / HC;
+    it.b = hsb / (G.Hkv * G.q_ns);
+    it.kvh = (hsb / G.q_ns) % G.Hkv;
+    it.s = hsb % G.q_ns;
+    const int grp_all = G.Hq / G.Hkv, hper = (grp_all + HC - 1) / HC;
+    it.grp = min(hper, grp_all - it.hc * hper);
+    it.h_base = it.kvh * grp_all + it.hc * hper;
+    it.head = it.h_base;
+    const int n0 = j * 2 * BM;
+    it.row0 = n0 + rank * BM;
+    // query rows that can see a key of the pair: key row r*qstep + qoff >= n0, and under
+    // a window r*qstep + qoff < n0 + 2*BM - 1 + window
+    it.lo = (n0 <= G.qoff ? 0 : (n0 - G.qoff + G.qstep - 1) / G.qstep) / BN;
+    int hi = (G.Lq - 1) / BN;
+    if (G.window > 0) hi = min(hi, ((n0 + 2 * BM - 2 + G.window - G.qoff) / G.qstep) / BN);
+    it.nst = hi - it.lo + 1;
+    it.T = it.nst > 0 ? it.grp * it.nst : 0;
+  } else {
+    idx -= 2 * P.nkv;
+    const int hp = P.head_pairs, rows = hp ? BM : 2 * BM, nh = hp ? G.Hq / 2 : G.Hq;
+    const int ntile = (G.Lq + rows - 1) / rows, per_rank = nh * G.q_ns * G.B;
+    const int mt = ntile - 1 - idx / per_rank, hsb = idx % per_rank;
+    it.b = hsb / (nh * G.q_ns);
+    it.s = hsb % G.q_ns;
+    const int hx = (hsb / G.q_ns) % nh;
+    it.head = hp ? 2 * hx + rank : hx;
+    it.kvh = it.head / (G.Hq / G.Hkv);
+    it.h_base = it.head;
+    it.grp = 1;
+    const int m0 = mt * rows;
+    it.row0 = hp ? m0 : m0 + rank * BM;
+    // key tiles some row of the pair sees
+    const int rq_first = m0 * G.qstep + G.qoff, rq_last = (min(m0 + rows, G.Lq) - 1) * G.qstep + G.qoff;
+    it.lo = G.window > 0 ? max(0, rq_first - G.window + 1) / BN : 0;
+    it.nst = min(rq_last, G.Lv - 1) / BN - it.lo + 1;
+    it.T = it.nst;
+  }
+  it.sk = it.s + G.kv_s0;
+  return it;
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_kernel(const __grid_constant__ Params P) {
   extern __shared__ uint8_t smem_raw[];
   {
     uint32_t dyn;
@@ -103,491 +220,476 @@ __global__ void __launch_bounds__(NTHREADS, 1) bwd256_kernel(const __grid_consta
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const SfaGeom& G = P.g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // linear grid, key tile slowest (the tiles with the most query tiles first); the two
-  // head-dim halves of a key tile are neighbours, then its head chunks
-  const int HC = P.hchunks;
-  const int per_tile = 2 * HC * G.Hkv * G.q_ns * G.B;
-  const int j = (int)blockIdx.x / per_tile;
-  const int rem = (int)blockIdx.x % per_tile;
-  const int c = rem & 1, hc = (rem >> 1) % HC, hsb = (rem >> 1) / HC;
-  const int o = c ^ 1;
-  const int n0 = j * BK;
-  const int b = hsb / (G.Hkv * G.q_ns), kvh = (hsb / G.q_ns) % G.Hkv, s = hsb % G.q_ns;
-  const int sk = s + G.kv_s0;  // stream of the key problem
-  // this CTA's query heads: chunk hc of the group's grp heads
-  const int grp_all = G.Hq / G.Hkv, hper = (grp_all + HC - 1) / HC;
-  const int grp = min(hper, grp_all - hc * hper);  // heads of this chunk (>= 1)
-  const int h_base = kvh * grp_all + hc * hper;
-  // query rows that can see a key of the tile: key row r*qstep + qoff >= n0, and under
-  // a window r*qstep + qoff < n0 + BK - 1 + window
-  const int i_lo = (n0 <= G.qoff ? 0 : (n0 - G.qoff + G.qstep - 1) / G.qstep) / BQ;
-  int i_hi = (G.Lq - 1) / BQ;
-  if (G.window > 0) i_hi = min(i_hi, ((n0 + BK - 2 + G.window - G.qoff) / G.qstep) / BQ);
-  const int nq = i_hi - i_lo + 1;
-  const int T = grp * nq;
-  const int Lqp = row_terms_pitch(G.Lq);
-  if (nq <= 0) {  // no query sees this key tile: its half of the dK and dV rows is zero
-    if (HC > 1) {  // this chunk's slice rows (its head-dim half) are zero
-      const size_t half = (size_t)G.B * G.q_ns * G.Lv * G.Hkv * DH;
-      for (int i = threadIdx.x; i < BK * (DHH / 4); i += NTHREADS) {
-        const int kr = n0 + i / (DHH / 4), c4 = i % (DHH / 4);
-        if (kr >= G.Lv) continue;
-        const long long wrow = ((((long long)b * G.q_ns + s) * G.Lv + kr) * G.Hkv + kvh) * DH + c * DHH + c4 * 4;
-        *reinterpret_cast<float4*>(P.dkv + (2 * hc) * half + wrow) = make_float4(0.f, 0.f, 0.f, 0.f);
-        *reinterpret_cast<float4*>(P.dkv + (2 * hc + 1) * half + wrow) = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      return;
-    }
-    for (int i = threadIdx.x; i < BK * (DHH / 8); i += NTHREADS) {
-      const int kr = n0 + i / (DHH / 8), cc = i % (DHH / 8);
+  const int rank = (int)(blockIdx.x & 1);  // = %cluster_ctarank
+  const Item it = make_item(P, (int)(blockIdx.x >> 1), rank);
+  const int kind = it.kind, T = it.T;
+  const size_t half = (size_t)G.B * G.q_ns * G.Lv * G.Hkv * DH;  // elements of a slice half
+  if (T <= 0) {  // no query sees these key tiles (the same for both CTAs): their rows are zero
+    for (int i = threadIdx.x; i < BM * (DH / 8); i += NTHREADS) {
+      const int kr = it.row0 + i / (DH / 8), c = i % (DH / 8);
       if (kr >= G.Lv) continue;
-      const long long orow = (((long long)b * G.nL + (long long)kr * G.rs + sk) * G.Hkv + kvh) * DH + c * DHH + cc * 8;
-      *reinterpret_cast<uint4*>(P.dk + orow) = make_uint4(0, 0, 0, 0);
-      *reinterpret_cast<uint4*>(P.dv + orow) = make_uint4(0, 0, 0, 0);
+      if (P.hchunks > 1) {
+        float* w = P.dkv + (2 * it.hc + (kind == kDK)) * half +
+                   ((((long long)it.b * G.q_ns + it.s) * G.Lv + kr) * G.Hkv + it.kvh) * DH + c * 8;
+        reinterpret_cast<float4*>(w)[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+        reinterpret_cast<float4*>(w)[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+      } else {
+        bf16* w = (kind == kDK ? P.dk : P.dv) +
+                  (((long long)it.b * G.nL + (long long)kr * G.rs + it.sk) * G.Hkv + it.kvh) * DH + c * 8;
+        *reinterpret_cast<uint4*>(w) = make_uint4(0, 0, 0, 0);
+      }
     }
     return;
   }
 
   if (threadIdx.x == 0) {
-    mbar_init(&sm.kv_full, 1);
+    for (int i = 0; i < NSLOT_DV; ++i) {
+      mbar_init(&sm.full[i], 1);
+      mbar_init(&sm.empty[i], 1);
+    }
+    mbar_init(&sm.a1_full, 1);
+    mbar_init(&sm.a2_full, 1);
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&sm.q_full[i], 1);
-      mbar_init(&sm.qc_empty[i], 1);
       mbar_init(&sm.s_full[i], 1);
-      mbar_init(&sm.dp_full[i], 1);
-      mbar_init(&sm.dq_full[i], 1);
-      mbar_init(&sm.s_init[i], 256);
-      mbar_init(&sm.dp_init[i], 256);
-      mbar_init(&sm.dv_done[i], 1);
-      mbar_init(&sm.dk_done[i], 1);
+      mbar_init(&sm.term_full[i], 1);
+      mbar_init(&sm.term_empty[i], 8);  // the CTA's softmax warps
+      mbar_init(&sm.p_full[i], 16);  // one arrival per softmax warp of the pair
     }
-    mbar_init(&sm.qo_empty, 1);
-    mbar_init(&sm.do_full, 1);
-    mbar_init(&sm.do_empty, 2);  // dV_c(t) and dP(t) both read dO(t)
-    for (int i = 0; i < 4; ++i) {
-      mbar_init(&sm.pa_part[i], 128);
-      mbar_init(&sm.pb_part[i], 128);
-    }
-    mbar_init(&sm.ds_free, 256);
-    mbar_init(&sm.kv_done, 1);
-    mbar_init(&sm.drain, 3);
+    mbar_init(&sm.s_empty, 16);
+    mbar_init(&sm.dp_full, 1);
+    mbar_init(&sm.out_done, 1);
     sm.abort = 0;
     fence_mbar_init();
   }
   if (warp == 0) {
-    tmem_alloc(&sm.tmem_base, 512);
-    tmem_relinquish();
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&sm.tmem_base)),
+                 "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // both CTAs' barriers are initialised and their TMEM is allocated
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
   volatile int* abort = &sm.abort;
+  const int nslot = kind == kDV ? NSLOT_DV : NSLOT;
+  bf16* const ring0 = kind == kDV ? sm.a2 : sm.ring[0];  // a2 and ring are adjacent
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      tma_prefetch(&P.tm_q);
-      tma_prefetch(&P.tm_do);
-      tma_prefetch(&P.tm_k);
-      tma_prefetch(&P.tm_v);
-      mbar_arrive_expect_tx(&sm.kv_full, 2 * BK * DH * 2);
-      for (int cc = 0; cc < DH / 64; ++cc) {
-        tma_load_5d(sm.k + cc * BK * 64, &P.tm_k, &sm.kv_full, cc * 64, kvh, sk, n0, b);
-        tma_load_5d(sm.v + cc * BK * 64, &P.tm_v, &sm.kv_full, cc * 64, kvh, sk, n0, b);
-      }
-      int nq_issued = 0, ndo_issued = 0;
-      // the query tile t: its other half once S^T(t-1)'s first k-steps are done, its own
-      // half into qc[t&1] once dK_c(t-2) is done; dO(t) once dV_c(t-1) and dP(t-1) are
-      for (int t = 0; t < T; ++t) {
-        const int h = h_base + t / nq, q0 = (i_lo + t % nq) * BQ;
-        const int qb = t & 1;
-        if (t >= 1 && !mbar_wait(&sm.qo_empty, (t - 1) & 1, abort, P.status)) break;
-        if (t >= 2 && !mbar_wait(&sm.qc_empty[qb], ((t - 2) >> 1) & 1, abort, P.status)) break;
-        mbar_arrive_expect_tx(&sm.q_full[qb], BQ * DH * 2 + 2 * BQ * 4);
-        for (int cc = 0; cc < 2; ++cc) {
-          tma_load_5d(sm.qo + cc * BQ * 64, &P.tm_q, &sm.q_full[qb], o * DHH + cc * 64, h, s, q0, b);
-          tma_load_5d(sm.qc[qb] + cc * BQ * 64, &P.tm_q, &sm.q_full[qb], c * DHH + cc * 64, h, s, q0, b);
-        }
-        const long long off = (((long long)b * G.Hq + h) * G.q_ns + s) * Lqp + q0;
-        bulk_load(sm.nlse2[qb], P.lse2 + off, BQ * 4, &sm.q_full[qb]);
-        bulk_load(sm.ndelta[qb], P.delta + off, BQ * 4, &sm.q_full[qb]);
-        ++nq_issued;
-        if (t >= 1 && !mbar_wait(&sm.do_empty, (t - 1) & 1, abort, P.status)) break;
-        mbar_arrive_expect_tx(&sm.do_full, BQ * DH * 2);
-        for (int cc = 0; cc < DH / 64; ++cc)
-          tma_load_5d(sm.dO + cc * BQ * 64, &P.tm_do, &sm.do_full, cc * 64, h, s, q0, b);
-        ++ndo_issued;
-      }
-      // every copy this thread started lands before the CTA may exit
-      mbar_drain(&sm.kv_full, 0);
-      for (int t = max(0, nq_issued - 2); t < nq_issued; ++t) mbar_drain(&sm.q_full[t & 1], (t >> 1) & 1);
-      if (ndo_issued > 0) mbar_drain(&sm.do_full, (ndo_issued - 1) & 1);
-    }
-  } else if (warp == 1 || warp == kWarpSP || warp == kWarpDQ) {
-    // ------------------------------------------------------------ MMA issuers
-    if (lane == 0 || warp != 1) {  // issuer X: one lane; the others: the whole warp, elected lanes issue
-      constexpr uint32_t idSP = idesc_bf16(128, BQ, 0, 0);   // S^T, dP^T: A = K / V, B = Q / dO (K-major)
-      constexpr uint32_t idKV = idesc_bf16(128, DHH, 0, 1);  // dV_c, dK_c: A in TMEM, B = dO / Q half, MN-major
-      constexpr uint32_t idQ = idesc_bf16(128, BQ, 1, 1);    // dQ_c^T: A = K half MN-major, B = dS^T MN-major
-      // Descriptors encoded once; a k-step adds its byte offset / 16 (shared addresses
-      // stay below 256 KB).  K-major: 32 bytes per k-step inside a 64-column block; a
-      // block is 16 KB for the 128-row K / V tiles and 8 KB for the 64-row query tiles.
-      // MN-major: 16 rows of 128 bytes per k-step; LBO = the stride of 64-column blocks.
-      auto kb = [](int kk) { return (uint64_t)((kk >> 2) * (BK * 128 / 16) + (kk & 3) * 2); };  // 128-row blocks
-      auto qb = [](int kk) { return (uint64_t)((kk >> 2) * (BQ * 128 / 16) + (kk & 3) * 2); };  // 64-row blocks
-      auto moff = [](int kk) { return (uint64_t)(kk * 16 * 128 / 16); };
+      const CUtensorMap *tA1 = kind == kDQ ? &P.tm_q : &P.tm_k, *tA2 = kind == kDQ ? &P.tm_do : &P.tm_v;
+      const CUtensorMap* tB1 = kind == kDQ ? &P.tm_k : &P.tm_q;
+      const CUtensorMap* tB2 = kind == kDQ ? &P.tm_v : &P.tm_do;
+      const CUtensorMap* tB3 = kind == kDV ? &P.tm_do : tB1;
+      tma_prefetch(tA1);
+      tma_prefetch(tA2);
+      tma_prefetch(tB1);
+      tma_prefetch(tB2);
+      const int ahead = kind == kDQ ? it.head : it.kvh, astr = kind == kDQ ? it.s : it.sk;
+      const int bstr = kind == kDQ ? it.sk : it.s;
+      auto load_a = [&](bf16* dst, const CUtensorMap* tm, uint64_t* bar) {
+        if (rank == 0) mbar_arrive_expect_tx(bar, 2 * BM * DH * 2);
+        const uint32_t lb = lead_addr(bar);
+        for (int c = 0; c < DH / 64; ++c)
+          for (int r = 0; r < BM / PR; ++r)
+            tma_load_pair(dst + c * BM * 64 + r * PR * 64, tm, lb, c * 64, ahead, astr, it.row0 + r * PR, it.b);
+      };
+      int terms_issued = 0;
+      int slot = 0, ph = 1;  // empty-barrier phase: the first lap does not wait
       bool ok = true;
-      if (warp == 1) {
-        // ---- issuer X: dV_c(t) and dK_c(t), one 16-query quarter at a time
-        const uint64_t doM = sdesc_sw128(smem_u32(sm.dO + c * 2 * BQ * 64), BQ * 128, 1024);  // dO[:, c]
-        const uint64_t qcM0 = sdesc_sw128(smem_u32(sm.qc[0]), BQ * 128, 1024),
-                       qcM1 = sdesc_sw128(smem_u32(sm.qc[1]), BQ * 128, 1024);
-        for (int t = 0; ok && t < T; ++t) {
-          const int p = t & 1;
-          const uint64_t qcM = p ? qcM1 : qcM0;
-          // dO(t) has landed (the S / dP issuer waits for it only before dP(t), which may
-          // come after phase A(t) has released P^T(t) here)
-          if (!mbar_wait(&sm.do_full, t & 1, abort, P.status)) { ok = false; break; }
-          for (int u = 0; u < 4; ++u) {
-            if (!mbar_wait(&sm.pa_part[u], t & 1, abort, P.status)) { ok = false; break; }
-            tc_fence_after();
-            tc_mma_ts(tmem + COL_DV, tmem + col_s(p) + u * 8, doM + moff(u), idKV, (t > 0 || u > 0) ? 1u : 0u);
-          }
-          if (!ok) break;
-          tc_commit(&sm.do_empty);
-          tc_commit(&sm.dv_done[p]);  // dQ_c^T(t) may land over P^T(t) in RS(p)
-          for (int u = 0; u < 4; ++u) {
-            if (!mbar_wait(&sm.pb_part[u], t & 1, abort, P.status)) { ok = false; break; }
-            tc_fence_after();
-            tc_mma_ts(tmem + COL_DK, tmem + col_d(p) + u * 8, qcM + moff(u), idKV, (t > 0 || u > 0) ? 1u : 0u);
-          }
-          if (!ok) break;
-          tc_commit(&sm.qc_empty[p]);
-          tc_commit(&sm.dk_done[p]);  // RD(p) free for the dP'^T(t+2) pre-fill
-        }
-        tc_commit(&sm.kv_done);
-        tc_commit(&sm.drain);
-      } else if (warp == kWarpSP) {
-        // ---- S^T(t) into RS(p), dP^T(t) into RD(p), as soon as their operands and
-        // pre-filled regions are ready
-        const uint64_t kK = sdesc_sw128(smem_u32(sm.k), 16, 1024), vK = sdesc_sw128(smem_u32(sm.v), 16, 1024);
-        const uint64_t qoK = sdesc_sw128(smem_u32(sm.qo), 16, 1024);
-        const uint64_t qcK0 = sdesc_sw128(smem_u32(sm.qc[0]), 16, 1024), qcK1 = sdesc_sw128(smem_u32(sm.qc[1]), 16, 1024);
-        const uint64_t doK = sdesc_sw128(smem_u32(sm.dO), 16, 1024);
-        ok = __all_sync(0xffffffffu, mbar_wait(&sm.kv_full, 0, abort, P.status));
-        for (int t = 0; ok && t < T; ++t) {
-          const int p = t & 1, ph = (t >> 1) & 1;
-          if (!__all_sync(0xffffffffu, mbar_wait(&sm.q_full[p], ph, abort, P.status)) ||
-              !__all_sync(0xffffffffu, mbar_wait(&sm.s_init[p], ph, abort, P.status))) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          // the other half's 8 k-steps first: its Q half is then released for tile t+1
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk) tc_mma_ss_w(tmem + col_s(p), kK + kb(8 * o + kk), qoK + qb(kk), idSP, 1u);
-          tc_commit_w(&sm.qo_empty);
-          const uint64_t qcK = p ? qcK1 : qcK0;
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk) tc_mma_ss_w(tmem + col_s(p), kK + kb(8 * c + kk), qcK + qb(kk), idSP, 1u);
-          tc_commit_w(&sm.s_full[p]);
-          if (!__all_sync(0xffffffffu, mbar_wait(&sm.do_full, t & 1, abort, P.status)) ||
-              !__all_sync(0xffffffffu, mbar_wait(&sm.dp_init[p], ph, abort, P.status))) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-#pragma unroll
-          for (int kk = 0; kk < DH / 16; ++kk) tc_mma_ss_w(tmem + col_d(p), vK + kb(kk), doK + qb(kk), idSP, 1u);
-          tc_commit_w(&sm.dp_full[p]);
-          tc_commit_w(&sm.do_empty);  // with issuer X's arrival after dV_c(t)
-        }
-        tc_commit_w(&sm.drain);
-      } else {
-        // ---- dQ_c^T(t) into RS(p): dS^T(t) complete in smem, P^T(t) consumed there
-        const uint64_t kcM = sdesc_sw128(smem_u32(sm.k + c * 2 * BK * 64), BK * 128, 1024);  // K[:, c]
-        const uint64_t dsM = sdesc_sw128(smem_u32(sm.ds), BK * 128, 1024);
-        for (int t = 0; ok && t < T; ++t) {
-          const int p = t & 1, ph = (t >> 1) & 1;
-          if (!__all_sync(0xffffffffu, mbar_wait(&sm.pb_part[3], t & 1, abort, P.status)) ||
-              !__all_sync(0xffffffffu, mbar_wait(&sm.dv_done[p], ph, abort, P.status))) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-#pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk)
-            tc_mma_ss_w(tmem + col_s(p), kcM + moff(kk), dsM + moff(kk), idQ, kk > 0 ? 1u : 0u);
-          tc_commit_w(&sm.dq_full[p]);
-        }
-        tc_commit_w(&sm.drain);
-      }
-      // every MMA any issuer started completes before TMEM / smem are released
-      mbar_drain(&sm.drain, 0);
-    }
-  } else if (warp < 6) {
-    // ------------------------------------------------------------ softmax
-    const int q4 = warp & 3;
-    const int row = q4 * 32 + lane;  // TMEM lane
-    const int kr = n0 + row;
-    const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16);
-    const float c2 = P.scale_log2;
-    uint8_t* dsrow = reinterpret_cast<uint8_t*>(sm.ds) + row * 128;
-    const uint64_t c2x2 = f2pack(c2, c2);
-    bool ok = true;
-    for (int t = 0; t < T; ++t) {
-      const int p = t & 1, ph = (t >> 1) & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(&sm.s_full[p], ph, abort, P.status))) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      // ---- phase A: P^T = exp2(c2 S'^T), packed bf16 over the first 32 columns of RS(p);
-      // four 16-column chunks, the loads of chunk u+1 in flight while chunk u is computed,
-      // each chunk published (stores landed) so its dV k-step may start
-      {
-        uint32_t sbuf[2][16];
-        tmem_ld16(tl + col_s(p), sbuf[0]);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          uint32_t* sr = sbuf[u & 1];
-          tmem_ld_wait();
-          if (u + 1 < 4) tmem_ld16(tl + col_s(p) + 16 * (u + 1), sbuf[(u + 1) & 1]);
-          float x[16];
-#pragma unroll
-          for (int e = 0; e < 16; e += 2)
-            f2unpack(fmul2(f2pack(__uint_as_float(sr[e]), __uint_as_float(sr[e + 1])), c2x2), x[e], x[e + 1]);
-          uint32_t pp[8];
-#pragma unroll
-          for (int e = 0; e < 16; e += 2) pp[e >> 1] = cvt_bf16x2(ex2_approx(x[e]), ex2_approx(x[e + 1]));
-          tmem_st8(tl + col_s(p) + 8 * u, pp);
-          tmem_st_wait();
-          tc_fence_before();
-          mbar_arrive(&sm.pa_part[u]);
-        }
-      }
-      if (!__all_sync(0xffffffffu, mbar_wait(&sm.dp_full[p], ph, abort, P.status))) {
-        ok = false;
-        break;
-      }
-      // the dQ staging of tile t-1 (over the dS^T buffer) has been read by its reduces
-      if (t > 0 && !__all_sync(0xffffffffu, mbar_wait(&sm.ds_free, (t - 1) & 1, abort, P.status))) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      // ---- phase B: dS^T = P^T dP'^T, packed bf16 into RD(p) and into shared memory
-      // for dQ_c^T(t)
-      {
-        uint32_t dbuf[2][16], pbuf[2][8];
-        tmem_ld16(tl + col_d(p), dbuf[0]);
-        tmem_ld8(tl + col_s(p), pbuf[0]);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          uint32_t *dr = dbuf[u & 1], *pr = pbuf[u & 1];
-          tmem_ld_wait();
-          if (u + 1 < 4) {
-            tmem_ld16(tl + col_d(p) + 16 * (u + 1), dbuf[(u + 1) & 1]);
-            tmem_ld8(tl + col_s(p) + 8 * (u + 1), pbuf[(u + 1) & 1]);
-          }
-          uint32_t dd[8];
-#pragma unroll
-          for (int e = 0; e < 16; e += 2)
-            dd[e >> 1] = mul_bf16x2(pr[e >> 1], cvt_bf16x2(__uint_as_float(dr[e]), __uint_as_float(dr[e + 1])));
-          tmem_st8(tl + col_d(p) + 8 * u, dd);
-          // dS^T row -> shared memory: 16-byte units 2u, 2u+1 of this key row's 128 bytes
-#pragma unroll
-          for (int kx = 0; kx < 2; ++kx)
-            *reinterpret_cast<uint4*>(dsrow + (((2 * u + kx) ^ (row & 7)) << 4)) =
-                make_uint4(dd[4 * kx], dd[4 * kx + 1], dd[4 * kx + 2], dd[4 * kx + 3]);
-          if (u == 3) fence_async_smem();
-          tmem_st_wait();
-          tc_fence_before();
-          mbar_arrive(&sm.pb_part[u]);
-        }
-      }
-    }
-    // epilogue: this key row's half of dV, then of dK (scaled); with head chunks, into
-    // this chunk's fp32 workspace slice instead
-    if (ok && __all_sync(0xffffffffu, mbar_wait(&sm.kv_done, 0, abort, P.status))) {
-      tc_fence_after();
-      const long long orow = (((long long)b * G.nL + (long long)kr * G.rs + sk) * G.Hkv + kvh) * DH + c * DHH;
-      const size_t half = (size_t)G.B * G.q_ns * G.Lv * G.Hkv * DH;
-      const long long wrow = ((((long long)b * G.q_ns + s) * G.Lv + kr) * G.Hkv + kvh) * DH + c * DHH;
+      // a unit: two pieces.  as_n: B of S / dP (this CTA's 64 rows, both halves of the
+      // head dim); else B of the output GEMM (all 128 rows, this CTA's head-dim half)
+      auto load_unit = [&](const CUtensorMap* tm, int t, bool as_n) {
+        const int hd = kind == kDQ ? it.kvh : it.h_base + t / it.nst;
+        const int r0 = (it.lo + (kind == kDQ ? t : t % it.nst)) * BN;
 #pragma unroll 1
-      for (int cc = 0; cc < 2 * DHH / 32; ++cc) {
-        const int which = cc >= DHH / 32;
-        const float mul = which ? P.scale : 1.f;
-        bf16* dst = (which ? P.dk : P.dv) + orow + (cc % (DHH / 32)) * 32;
-        const uint32_t col = (which ? COL_DK : COL_DV) + (cc % (DHH / 32)) * 32;
-        uint32_t ov[32];
-        tmem_ld32(tl + col, ov);
-        tmem_ld_wait();
-        if (HC > 1) {
-          if (kr < G.Lv) {
-            float* wdst = P.dkv + (2 * hc + which) * half + wrow + (cc % (DHH / 32)) * 32;
-#pragma unroll
-            for (int e = 0; e < 32; e += 4)
-              *reinterpret_cast<float4*>(wdst + e) =
-                  make_float4(__uint_as_float(ov[e]) * mul, __uint_as_float(ov[e + 1]) * mul,
-                              __uint_as_float(ov[e + 2]) * mul, __uint_as_float(ov[e + 3]) * mul);
+        for (int p = 0; p < 2 && ok; ++p) {
+          if (!mbar_wait(&sm.empty[slot], ph, abort, P.status)) {
+            ok = false;
+            return;
           }
-        } else if (kr < G.Lv) {
-#pragma unroll
-          for (int e = 0; e < 32; e += 8) {
-            uint4 w;
-            w.x = cvt_bf16x2(__uint_as_float(ov[e + 0]) * mul, __uint_as_float(ov[e + 1]) * mul);
-            w.y = cvt_bf16x2(__uint_as_float(ov[e + 2]) * mul, __uint_as_float(ov[e + 3]) * mul);
-            w.z = cvt_bf16x2(__uint_as_float(ov[e + 4]) * mul, __uint_as_float(ov[e + 5]) * mul);
-            w.w = cvt_bf16x2(__uint_as_float(ov[e + 6]) * mul, __uint_as_float(ov[e + 7]) * mul);
-            *reinterpret_cast<uint4*>(dst + e) = w;
+          if (rank == 0) mbar_arrive_expect_tx(&sm.full[slot], 2 * PR * PC * 2);
+          const uint32_t lb = lead_addr(&sm.full[slot]);
+          bf16* dst = ring0 + slot * (PR * PC);
+          const int row = as_n ? r0 + rank * PR : r0 + p * PR, col = as_n ? p * PC : rank * PC;
+          tma_load_pair(dst, tm, lb, col, hd, bstr, row, it.b);
+          tma_load_pair(dst + PR * 64, tm, lb, col + 64, hd, bstr, row, it.b);
+          if (++slot == nslot) {
+            slot = 0;
+            ph ^= 1;
           }
         }
+      };
+      // the row terms of step t (DK, DV), into the buffer that step t-2 has read
+      auto load_terms = [&](int t) {
+        if (t >= 2 && !mbar_wait(&sm.term_empty[t & 1], ((t >> 1) - 1) & 1, abort, P.status)) {
+          ok = false;
+          return;
+        }
+        const long long off = (((long long)it.b * G.Hq + it.h_base + t / it.nst) * G.q_ns + it.s) *
+                                  row_terms_pitch(G.Lq) + (long long)(it.lo + t % it.nst) * BN;
+        mbar_arrive_expect_tx(&sm.term_full[t & 1], kind == kDK ? 2 * BN * 4 : BN * 4);
+        bulk_load(sm.nlse2[t & 1], P.lse2 + off, BN * 4, &sm.term_full[t & 1]);
+        if (kind == kDK) bulk_load(sm.ndelta[t & 1], P.delta + off, BN * 4, &sm.term_full[t & 1]);
+        terms_issued = t + 1;
+      };
+      load_a(sm.a1, tA1, &sm.a1_full);
+      load_unit(tB1, 0, true);
+      if (kind != kDQ) load_terms(0);
+      if (kind == kDV) {
+        for (int t = 0; ok && t < T; ++t) {
+          if (t + 1 < T) load_unit(tB1, t + 1, true);
+          if (ok && t + 1 < T) load_terms(t + 1);
+          if (ok) load_unit(tB3, t, false);
+        }
+      } else {
+        load_a(sm.a2, tA2, &sm.a2_full);
+        load_unit(tB2, 0, true);
+        if (ok && T > 1) load_unit(tB1, 1, true);
+        for (int t = 0; ok && t < T; ++t) {
+          load_unit(tB3, t, false);
+          if (ok && kind == kDK && t + 1 < T) load_terms(t + 1);
+          if (ok && t + 1 < T) load_unit(tB2, t + 1, true);
+          if (ok && t + 2 < T) load_unit(tB1, t + 2, true);
+        }
       }
+      for (int t = max(0, terms_issued - 2); t < terms_issued; ++t) mbar_drain(&sm.term_full[t & 1], (t >> 1) & 1);
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issuer (first CTA)
+    if (rank == 0) {
+      constexpr uint32_t idS = idesc_bf16(2 * BM, BN, 0, 0);  // S, dP: both operands K-major
+      constexpr uint32_t idO = idesc_bf16(2 * BM, DH, 0, 1);  // output: A in TMEM, B MN-major
+      // descriptors encoded once; a block, slot or k-step adds its byte offset / 16
+      const uint64_t a1d = sdesc_sw128(smem_u32(sm.a1), 16, 1024), a2d = sdesc_sw128(smem_u32(sm.a2), 16, 1024);
+      const uint64_t bK = sdesc_sw128(smem_u32(ring0), 16, 1024);          // pieces K-major
+      const uint64_t bM = sdesc_sw128(smem_u32(ring0), PR * 128, 1024);    // pieces MN-major
+      int slot = 0, ph = 0;
+      auto wait_w = [&](uint64_t* bar, int par) -> bool {
+        if (!__all_sync(0xffffffffu, mbar_wait(bar, par & 1, abort, P.status))) return false;
+        tc_fence_after();
+        return true;
+      };
+      auto next_piece = [&]() {
+        if (++slot == nslot) {
+          slot = 0;
+          ph ^= 1;
+        }
+      };
+      // D[256 x 128] = A B^T over the head dim, then a signal that it is complete
+      auto gemm_n = [&](uint32_t col, uint64_t ad, uint64_t* done) -> bool {
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          if (!wait_w(&sm.full[slot], ph)) return false;
+          const uint64_t bd = bK + (uint64_t)(slot * (PR * PC * 2 / 16));
+#pragma unroll
+          for (int k8 = 0; k8 < 8; ++k8) {
+            const int kk = p * 8 + k8;
+            mma2_ss(tmem + col, ad + (uint64_t)((kk >> 2) * (BM * 128 / 16) + (kk & 3) * 2),
+                    bd + (uint64_t)((k8 >> 2) * (PR * 128 / 16) + (k8 & 3) * 2), idS, kk > 0 ? 1u : 0u);
+          }
+          if (p == 1) commit2(done);
+          commit2(&sm.empty[slot]);
+          next_piece();
+        }
+        return true;
+      };
+      // out[256 x 256] += A[tmem] B over the 128 streamed rows.  The pieces are waited for
+      // before A (each wait costs about 100 cycles of a chain that ends with A).
+      auto gemm_out = [&](uint32_t acol, uint64_t* a_full, int a_par, bool acc0) -> bool {
+        const int s0 = slot;
+        if (!wait_w(&sm.full[slot], ph)) return false;
+        next_piece();
+        const int s1 = slot;
+        if (!wait_w(&sm.full[slot], ph) || !wait_w(a_full, a_par)) return false;
+        next_piece();
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          const uint64_t bd = bM + (uint64_t)((p ? s1 : s0) * (PR * PC * 2 / 16));
+#pragma unroll
+          for (int k4 = 0; k4 < 4; ++k4) {
+            const int kk = p * 4 + k4;
+            // P / dS: each 64-column half packed at the start of its own columns
+            mma2_ts(tmem + COL_OUT, tmem + acol + p * HB + k4 * 8, bd + (uint64_t)(k4 * 16 * 128 / 16), idO,
+                    (acc0 || kk > 0) ? 1u : 0u);
+          }
+          commit2(&sm.empty[p ? s1 : s0]);
+        }
+        return true;
+      };
+      bool ok = wait_w(&sm.a1_full, 0) && gemm_n(0, a1d, &sm.s_full[0]);
+      if (kind == kDV) {
+        for (int t = 0; ok && t < T; ++t) {
+          // S(t+1) over P^T(t-1), which out(t-1), issued before, has read
+          if (t + 1 < T) ok = gemm_n(((t + 1) & 1) * COL_D, a1d, &sm.s_full[(t + 1) & 1]);
+          ok = ok && gemm_out((t & 1) * COL_D, &sm.p_full[t & 1], t >> 1, t > 0);
+        }
+      } else {
+        ok = ok && wait_w(&sm.a2_full, 0) && gemm_n(COL_D, a2d, &sm.dp_full);
+        if (ok && T > 1) ok = wait_w(&sm.s_empty, 0) && gemm_n(0, a1d, &sm.s_full[0]);
+        for (int t = 0; ok && t < T; ++t) {
+          ok = gemm_out(COL_D, &sm.p_full[0], t, t > 0);
+          // dP(t+1) over dS(t), which out(t), issued before, has read
+          if (ok && t + 1 < T) ok = gemm_n(COL_D, a2d, &sm.dp_full);
+          if (ok && t + 2 < T) ok = wait_w(&sm.s_empty, t + 1) && gemm_n(0, a1d, &sm.s_full[0]);
+        }
+      }
+      // every MMA issued above completes before TMEM / smem are released
+      commit2(&sm.out_done);
+      mbar_drain(&sm.out_done, 0);
     }
   } else {
-    // ------------------------------------------------------------ pre-fills, dQ
-    // Pre-fill, query columns [32*hh, +32) of a region, this warp's TMEM lanes (key rows):
-    // -lse2/c2 of the query tile before its S^T MMA, -inf where the key row does not
-    // see the query (exp2 then gives P = 0 whatever the MMA adds); -delta before its
-    // dP^T MMA.  Tiles 0 and 1 are pre-filled up front; tile t+2 into the pair tile t
-    // frees: RS(p) once dQ_c^T(t) is read out of it (after its staging, which phase B
-    // of tile t+1 waits for), RD(p) once dK_c(t) has read dS^T(t).
-    // dQ_c^T: TMEM lane = head-dim column c*128 + 32*q4 + lane, this warp's 32 queries;
-    // staged as [16 queries][32 columns] fp32 (two rounds through this warp's 2 KB of
-    // the dS^T buffer) and added into the accumulator by TMA reduce.
-    const int hh = (warp - 6) >> 2;
-    const int q4 = warp & 3;
-    const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16);
-    float* stage = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(sm.ds) + (warp - 6) * 2048);
-    const float inv_c2 = 1.f / P.scale_log2;
-    const int kr = n0 + q4 * 32 + lane;  // key row of this thread's TMEM lane
-    auto s_values = [&](uint32_t* w, const float* src, int qm) {
-      const float4* s4 = reinterpret_cast<const float4*>(src + 32 * hh);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 x = s4[i];
-        w[4 * i] = __float_as_uint(x.x * inv_c2);
-        w[4 * i + 1] = __float_as_uint(x.y * inv_c2);
-        w[4 * i + 2] = __float_as_uint(x.z * inv_c2);
-        w[4 * i + 3] = __float_as_uint(x.w * inv_c2);
-      }
-      // masked where a pair can fall outside: the diagonal band, (LOCAL) the last query's
-      // window edge at or above the tile's first key, ragged tiles
-      const bool win_edge = WIN ? (qm + BQ - 1) * G.qstep + G.qoff - G.window >= n0 : G.window > 0;
-      if ((qm * G.qstep + G.qoff < n0 + BK) || win_edge || (n0 + BK > G.Lv) || (qm + BQ > G.Lq)) {
-        // key row kr sees the queries q in [vis_lo, vis_hi): q*qstep + qoff >= kr
-        // (causal), q < Lq, and for LOCAL q*qstep + qoff < kr + window
-        const int vis_lo = kr <= G.qoff ? 0 : (kr - G.qoff + G.qstep - 1) / G.qstep;
-        int vis_hi = G.Lq;
-        if (G.window > 0) {
-          const int e = kr + G.window - G.qoff;  // q*qstep < e
-          vis_hi = min(vis_hi, e <= 0 ? 0 : (e + G.qstep - 1) / G.qstep);
-        }
-        if (kr >= G.Lv) vis_hi = 0;
-        const int qb = qm + 32 * hh;
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (qb + i < vis_lo || qb + i >= vis_hi) w[i] = __float_as_uint(-INFINITY);
-      }
-    };
-    auto d_values = [&](uint32_t* w, const float* src) {  // dP'^T: -delta
-      const uint4* s4 = reinterpret_cast<const uint4*>(src + 32 * hh);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const uint4 x = s4[i];
-        w[4 * i] = x.x;
-        w[4 * i + 1] = x.y;
-        w[4 * i + 2] = x.z;
-        w[4 * i + 3] = x.w;
-      }
-    };
-    auto publish = [&](uint64_t* bar) {  // stores landed, then signal the MMA thread
-      tmem_st_wait();
+    // ------------------------------------------------------------ softmax / epilogue
+    // Two threads per stationary row (TMEM lane), each half hc of the 128 streamed columns.
+    const int q4 = warp & 3, hc = (warp - 2) >> 2;
+    const int r = it.row0 + q4 * 32 + lane;  // stationary row: query row (DQ) or key row (DK, DV)
+    const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16) + HB * hc;  // this thread's half
+    const float c2 = P.scale_log2;
+    const uint64_t c2x2 = f2pack(c2, c2);
+    const uint32_t lead_s_empty = lead_addr(&sm.s_empty);
+    const uint32_t lead_p[2] = {lead_addr(&sm.p_full[0]), lead_addr(&sm.p_full[1])};
+    auto publish = [&](uint32_t bar) {  // this warp's TMEM accesses are done: tell the issuer
       tc_fence_before();
-      mbar_arrive(bar);
-    };
-    auto tile_q0 = [&](int t) { return (i_lo + t % nq) * BQ; };
-    bool ok = true;
-    for (int t = 0; ok && t < 2 && t < T; ++t) {  // tiles 0 and 1: both region pairs
-      uint32_t w[32];
-      if (!__all_sync(0xffffffffu, mbar_wait(&sm.q_full[t], 0, abort, P.status))) {
-        ok = false;
-        break;
-      }
-      s_values(w, sm.nlse2[t], tile_q0(t));
-      tmem_st32(tl + col_s(t) + 32 * hh, w);
-      publish(&sm.s_init[t]);
-      d_values(w, sm.ndelta[t]);
-      tmem_st32(tl + col_d(t) + 32 * hh, w);
-      publish(&sm.dp_init[t]);
-    }
-    for (int t = 0; ok && t < T; ++t) {
-      const int p = t & 1, ph = (t >> 1) & 1;
-      const int h = h_base + t / nq, q0 = tile_q0(t);
-      const bool refill = t + 2 < T;
-      if (!__all_sync(0xffffffffu, mbar_wait(&sm.dq_full[p], ph, abort, P.status))) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      uint32_t v[32];
-      tmem_ld32(tl + col_s(p) + 32 * hh, v);
-      tmem_ld_wait();
-#pragma unroll
-      for (int r2 = 0; r2 < 2; ++r2) {
-        // the previous reduce from this warp's staging must have read it
-        if (lane == 0) bulk_wait_read0();
-        __syncwarp();
-        // query row 16*r2 + i of this warp's 32, head-dim column lane: 128-byte rows
-#pragma unroll
-        for (int i = 0; i < 16; ++i) stage[i * 32 + lane] = __uint_as_float(v[16 * r2 + i]);
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-          tma_reduce_add_5d(&P.tm_dq, stage, c * DHH + 32 * q4, h, s, q0 + 32 * hh + 16 * r2, b);
-          bulk_commit();
-        }
-      }
-      // the staging is read: phase B(t+1) may write dS^T(t+1) over it
-      if (lane == 0) bulk_wait_read0();
       __syncwarp();
-      mbar_arrive(&sm.ds_free);
-      if (refill) {
-        // RS(p) for S'^T(t+2): its row terms arrive with its query tile (after dK_c(t))
-        uint32_t w[32];
-        if (!__all_sync(0xffffffffu, mbar_wait(&sm.q_full[p], ph ^ 1, abort, P.status))) {
-          ok = false;
-          break;
+      if (lane == 0) arrive_lead(bar);
+    };
+    auto load_half = [&](uint32_t tcol, float* x) {
+#pragma unroll
+      for (int c = 0; c < HB / 32; ++c) tmem_ld32(tcol + c * 32, reinterpret_cast<uint32_t*>(x) + c * 32);
+      tmem_ld_wait();
+    };
+    // dS = P (dP - delta), packed bf16 over the first half of this thread's dP columns,
+    // all of them read before (the loads run one 16-column chunk ahead)
+    auto d_half = [&](const float* x, auto nd) {
+      uint32_t d[2][16];
+      tmem_ld16(tl + COL_D, d[0]);
+#pragma unroll
+      for (int c = 0; c < HB / 16; ++c) {
+        uint32_t* dc = d[c & 1];
+        tmem_ld_wait();
+        if (c + 1 < HB / 16) tmem_ld16(tl + COL_D + (c + 1) * 16, d[(c + 1) & 1]);
+        uint32_t pk[8];
+#pragma unroll
+        for (int e = 0; e < 16; e += 2) {
+          float y0, y1;
+          f2unpack(fmul2(fadd2(f2pack(__uint_as_float(dc[e]), __uint_as_float(dc[e + 1])), nd(c * 8 + (e >> 1))),
+                         f2pack(x[c * 16 + e], x[c * 16 + e + 1])),
+                   y0, y1);
+          pk[e >> 1] = cvt_bf16x2(y0, y1);
         }
-        s_values(w, sm.nlse2[p], tile_q0(t + 2));
-        tmem_st32(tl + col_s(p) + 32 * hh, w);
-        publish(&sm.s_init[p]);
+        tmem_st8(tl + COL_D + c * 8, pk);
       }
-      if (refill) {
-        // RD(p) for dP'^T(t+2) once dK_c(t) has read dS^T(t) there
-        uint32_t w[32];
-        if (!__all_sync(0xffffffffu, mbar_wait(&sm.dk_done[p], ph, abort, P.status))) {
+      tmem_st_wait();
+    };
+    bool ok = true;
+
+    if (kind == kDQ) {
+      const int rq = r * G.qstep + G.qoff;             // key row of this query
+      const int rq0 = it.row0 * G.qstep + G.qoff;      // ... of the tile's first query
+      const int rq1 = (it.row0 + BM - 1) * G.qstep + G.qoff;
+      float nl = -INFINITY, nd = 0.f;  // rows past Lq: P = 0
+      if (r < G.Lq) {
+        const long long off = (((long long)it.b * G.Hq + it.head) * G.q_ns + it.s) * row_terms_pitch(G.Lq) + r;
+        nl = P.lse2[off];
+        nd = P.delta[off];
+      }
+      const uint64_t nl2 = f2pack(nl, nl), nd2 = f2pack(nd, nd);
+      for (int t = 0; t < T; ++t) {
+        const int c0 = (it.lo + t) * BN + HB * hc;  // first key of this half
+        if (!__all_sync(0xffffffffu, mbar_wait(&sm.s_full[0], t & 1, abort, P.status))) {
           ok = false;
           break;
         }
         tc_fence_after();
-        d_values(w, sm.ndelta[p]);
-        tmem_st32(tl + col_d(p) + 32 * hh, w);
-        publish(&sm.dp_init[p]);
+        float x[HB];
+        load_half(tl, x);
+        publish(lead_s_empty);
+#pragma unroll
+        for (int e = 0; e < HB; e += 2) {
+          float a0, a1;
+          f2unpack(ffma2(f2pack(x[e], x[e + 1]), c2x2, nl2), a0, a1);
+          x[e] = ex2_approx(a0);
+          x[e + 1] = ex2_approx(a1);
+        }
+        // halves with a key past the first query's key row, at or below the last query's
+        // window edge, or past the end (keys there are zero, but exp2(-lse2) may overflow)
+        if (c0 + HB - 1 > rq0 || (G.window > 0 && c0 <= rq1 - G.window) || c0 + HB > G.Lv) {
+          const int hi = min(rq, G.Lv - 1) - c0, lo = G.window > 0 ? rq - G.window + 1 - c0 : 0;
+#pragma unroll
+          for (int e = 0; e < HB; ++e)
+            if (e > hi || e < lo) x[e] = 0.f;
+        }
+        if (!__all_sync(0xffffffffu, mbar_wait(&sm.dp_full, t & 1, abort, P.status))) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        d_half(x, [&](int) { return nd2; });
+        publish(lead_p[0]);
+      }
+    } else {
+      // DK, DV: this thread's key row r.  The streamed tile's row terms come through shared
+      // memory and are taken into registers before the MMA results they belong to are
+      // waited for: a broadcast load queues behind the MMAs' operand reads.
+      const int kr = r;
+      // key row kr sees the queries q in [vis_lo, vis_hi): q*qstep + qoff >= kr (causal),
+      // and for LOCAL q*qstep + qoff < kr + window.  Queries past Lq have -lse2 = -inf; a
+      // key row past Lv is not stored.
+      const int vis_lo = kr <= G.qoff ? 0 : (kr - G.qoff + G.qstep - 1) / G.qstep;
+      int vis_hi = G.Lq;
+      if (G.window > 0) {
+        const int e = kr + G.window - G.qoff;  // q*qstep < e
+        vis_hi = min(vis_hi, e <= 0 ? 0 : (e + G.qstep - 1) / G.qstep);
+      }
+      int qi = 0;  // query tile of the step within its head
+      for (int t = 0; t < T; ++t) {
+        const int qm = (it.lo + qi) * BN;
+        if (++qi == it.nst) qi = 0;
+        const int sb = kind == kDV ? (t & 1) : 0;
+        const uint32_t tS = tl + sb * COL_D;
+        if (!__all_sync(0xffffffffu, mbar_wait(&sm.term_full[t & 1], (t >> 1) & 1, abort, P.status))) {
+          ok = false;
+          break;
+        }
+        ulonglong2 tm[HB / 4];
+#pragma unroll
+        for (int e = 0; e < HB / 4; ++e) tm[e] = reinterpret_cast<const ulonglong2*>(sm.nlse2[t & 1] + HB * hc)[e];
+        if (!__all_sync(0xffffffffu, mbar_wait(&sm.s_full[sb], (kind == kDV ? t >> 1 : t) & 1, abort, P.status))) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        float x[HB];
+        load_half(tS, x);
+        if (kind == kDK) publish(lead_s_empty);
+#pragma unroll
+        for (int e = 0; e < HB; e += 2) {
+          float a0, a1;
+          f2unpack(ffma2(f2pack(x[e], x[e + 1]), c2x2, (e & 2) ? tm[e >> 2].y : tm[e >> 2].x), a0, a1);
+          x[e] = ex2_approx(a0);
+          x[e + 1] = ex2_approx(a1);
+        }
+        // the diagonal band and (LOCAL) tiles that reach the window edge of the first key
+        if (qm * G.qstep + G.qoff < it.row0 + BM ||
+            (G.window > 0 && (qm + BN - 1) * G.qstep + G.qoff - G.window >= it.row0)) {
+          const int lo = vis_lo - qm - HB * hc, hi = vis_hi - qm - HB * hc;
+#pragma unroll
+          for (int e = 0; e < HB; ++e)
+            if (e < lo || e >= hi) x[e] = 0.f;
+        }
+        if (kind == kDV) {
+#pragma unroll
+          for (int c = 0; c < HB / 32; ++c) {
+            uint32_t pk[16];
+#pragma unroll
+            for (int e = 0; e < 32; e += 2) pk[e >> 1] = cvt_bf16x2(x[c * 32 + e], x[c * 32 + e + 1]);
+            tmem_st16(tS + c * 16, pk);
+          }
+          tmem_st_wait();
+        } else {
+          const ulonglong2* nd4 = reinterpret_cast<const ulonglong2*>(sm.ndelta[t & 1] + HB * hc);
+          ulonglong2 td[HB / 4];
+#pragma unroll
+          for (int e = 0; e < HB / 8; ++e) td[e] = nd4[e];
+          if (!__all_sync(0xffffffffu, mbar_wait(&sm.dp_full, t & 1, abort, P.status))) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          d_half(x, [&](int e2) {
+            if (e2 < HB / 4 && !(e2 & 7)) {  // one chunk ahead of their use, in the registers the first half leaves
+#pragma unroll
+              for (int e = 0; e < 4; ++e) td[HB / 8 + (e2 >> 1) + e] = nd4[HB / 8 + (e2 >> 1) + e];
+            }
+            return (e2 & 1) ? td[e2 >> 1].y : td[e2 >> 1].x;
+          });
+        }
+        publish(lead_p[sb]);
+        if (lane == 0) mbar_arrive(&sm.term_empty[t & 1]);
       }
     }
-    if (lane == 0) bulk_wait0();
-    __syncwarp();
+
+    // epilogue: this thread's half (128 columns) of its row of the output
+    if (ok && __all_sync(0xffffffffu, mbar_wait(&sm.out_done, 0, abort, P.status))) {
+      tc_fence_after();
+      const uint32_t to = tmem + ((uint32_t)(q4 * 32) << 16) + COL_OUT + PC * hc;
+      const float mul = kind == kDV ? 1.f : P.scale;
+      const bool f32_out = kind == kDQ ? P.dq == nullptr : P.hchunks > 1;
+      const int nrow = kind == kDQ ? G.Lq : G.Lv;
+      if (f32_out) {
+        float* dst;
+        float m = mul;
+        if (kind == kDQ) {  // unscaled: sfa_bwd_finalize applies the scale
+          dst = P.dq_acc + (((long long)it.b * G.q_nL + (long long)r * G.q_rs + it.s) * G.Hq + it.head) * DH;
+          m = 1.f;
+        } else {
+          dst = P.dkv + (2 * it.hc + (kind == kDK)) * half +
+                ((((long long)it.b * G.q_ns + it.s) * G.Lv + r) * G.Hkv + it.kvh) * DH;
+        }
+        dst += PC * hc;
+#pragma unroll 1
+        for (int c = 0; c < PC / 32; ++c) {
+          uint32_t o[32];
+          tmem_ld32(to + c * 32, o);
+          tmem_ld_wait();
+          if (r < nrow) {
+#pragma unroll
+            for (int e = 0; e < 32; e += 4)
+              *reinterpret_cast<float4*>(dst + c * 32 + e) =
+                  make_float4(__uint_as_float(o[e]) * m, __uint_as_float(o[e + 1]) * m,
+                              __uint_as_float(o[e + 2]) * m, __uint_as_float(o[e + 3]) * m);
+          }
+        }
+      } else {
+        // rows leave through shared memory (A1 is no longer read): each thread writes its
+        // half row as bf16, 16-byte units XOR-swizzled by the row, then every store
+        // instruction of the warp writes 256-byte halves of two rows
+        constexpr int UPR = DH * 2 / 16;  // 16-byte units per row
+        uint8_t* stg = reinterpret_cast<uint8_t*>(sm.a1) + q4 * (32 * DH * 2);
+#pragma unroll 2
+        for (int c = 0; c < PC / 32; ++c) {
+          uint32_t o[32];
+          tmem_ld32(to + c * 32, o);
+          tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 32; e += 8) {
+            uint4 w;
+            w.x = cvt_bf16x2(__uint_as_float(o[e + 0]) * mul, __uint_as_float(o[e + 1]) * mul);
+            w.y = cvt_bf16x2(__uint_as_float(o[e + 2]) * mul, __uint_as_float(o[e + 3]) * mul);
+            w.z = cvt_bf16x2(__uint_as_float(o[e + 4]) * mul, __uint_as_float(o[e + 5]) * mul);
+            w.w = cvt_bf16x2(__uint_as_float(o[e + 6]) * mul, __uint_as_float(o[e + 7]) * mul);
+            const int u = hc * (UPR / 2) + c * 4 + e / 8;
+            *reinterpret_cast<uint4*>(stg + lane * (DH * 2) + ((u ^ (lane & 7)) << 4)) = w;
+          }
+        }
+        __syncwarp();
+        bf16* base;
+        long long rstride;  // elements between rows
+        if (kind == kDQ) {
+          base = P.dq + (((long long)it.b * G.q_nL + it.s) * G.Hq + it.head) * DH;
+          rstride = (long long)G.q_rs * G.Hq * DH;
+        } else {
+          base = (kind == kDK ? P.dk : P.dv) + (((long long)it.b * G.nL + it.sk) * G.Hkv + it.kvh) * DH;
+          rstride = (long long)G.rs * G.Hkv * DH;
+        }
+        const int r0 = it.row0 + q4 * 32, u = hc * (UPR / 2) + (lane & 15);
+#pragma unroll 8
+        for (int i = lane >> 4; i < 32; i += 2)
+          if (r0 + i < nrow)
+            *reinterpret_cast<uint4*>(base + (long long)(r0 + i) * rstride + u * 8) =
+                *reinterpret_cast<const uint4*>(stg + i * (DH * 2) + ((u ^ (i & 7)) << 4));
+      }
+    }
   }
 
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // neither CTA's barriers or TMEM are used any more
   if (warp == 0) {
-    __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512) : "memory");
   }
 }
 // Head chunks: dv / dk rows (bf16) from the chunks' fp32 partial sums, added in chunk
@@ -623,41 +725,105 @@ __global__ void __launch_bounds__(256) dkv_finalize_kernel(const float* __restri
     *reinterpret_cast<uint4*>((which ? dk : dv) + orow) = w;
   }
 }
+
+// DK / DV items of one chunk count.
+static long long key_items(const SfaGeom& g) {
+  return (long long)((g.Lv + 2 * BM - 1) / (2 * BM)) * g.Hkv * g.q_ns * g.B;
+}
+
+// Query-head chunks of the DK and DV items: the count with the least estimated time over
+// the chip's 76 CTA pairs, as the larger of a pair's share of all items and the longest
+// item (DK of the key pair with the most query tiles), plus the finalize pass where there
+// are chunks.  In units of 1000 cycles, measured at L = 4096: a step of DK, DV and DQ 4.1,
+// 2.5 and 3.8, an item's fixed part 10, the finalize pass 8 and its traffic (8 bytes
+// written and read per element and chunk at about 3.4 KB per cycle).  `room`: slices of
+// partial sums there is space for.  (One chunk too many costs little on long items, but
+// three sequences of 98 positions, fwd + bwd: 63 us with 12 chunks, two waves of short items, 50 us with 4.)
+static int head_chunks(const SfaGeom& g, long long room, long long ndq) {
+  const int grp = g.Hq / g.Hkv;
+  const long long items = key_items(g);
+  constexpr int kPairs = kSmCount / 2;
+  if (grp < 2 || room < 2 || items >= 2 * kPairs) return 1;
+  // query tiles per head that each key pair streams (fewer than 2 * kPairs pairs)
+  const int npair = (g.Lv + 2 * BM - 1) / (2 * BM);
+  double sum = 0, most = 0;
+  for (int j = 0; j < npair; ++j) {
+    const int n0 = j * 2 * BM;
+    const int lo = (n0 <= g.qoff ? 0 : (n0 - g.qoff + g.qstep - 1) / g.qstep) / BN;
+    int hi = (g.Lq - 1) / BN;
+    if (g.window > 0 && n0 + 2 * BM - 2 + g.window - g.qoff < (hi + 1) * BN * g.qstep)
+      hi = (n0 + 2 * BM - 2 + g.window - g.qoff) / g.qstep / BN;
+    const double nst = hi >= lo ? hi - lo + 1 : 0;
+    sum += nst;
+    most = nst > most ? nst : most;
+  }
+  const double per = (double)items / npair;  // items of one key pair
+  // DQ: as many row-tile products as DK, two row tiles to an item
+  const double dq = ndq * 10.0 + 3.8 * sum * per * grp;
+  int best = 1;
+  double best_cost = 0;
+  for (int hs = 1; hs <= grp && hs <= room; ++hs) {
+    const int hper = (grp + hs - 1) / hs;
+    if ((grp + hper - 1) / hper != hs) continue;  // another count gives the same chunks
+    const double total = dq + 2.0 * items * hs * 10.0 + 6.6 * sum * per * grp;
+    const double longest = 10.0 + 4.1 * hper * most;
+    const double share = total / kPairs;
+    double cost = share > longest ? share : longest;
+    if (hs > 1) cost += 8.0 + 16.0 * hs * g.B * g.q_ns * (double)g.Lv * g.Hkv * DH / 3.4e6;
+    if (best_cost == 0 || cost < best_cost) {
+      best = hs;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
 }  // namespace tcbwd256
 
-cudaError_t launch_sfa_bwd_main_tc256(const void* q, const void* k, const void* v, const void* dout, void* dk,
-                                      void* dv, const float* lse2_ws, const float* delta_ws, float* dq_ws,
+// dq_out: bf16 dQ (scaled); null: unscaled fp32 dQ into dq_ws.  With dq_out the space of
+// dq_ws is free and holds the chunks' partial sums when it is larger than dkv_ws.
+cudaError_t launch_sfa_bwd_main_tc256(const void* q, const void* k, const void* v, const void* dout, void* dq_out,
+                                      void* dk, void* dv, const float* lse2_ws, const float* delta_ws, float* dq_ws,
                                       float* dkv_ws, const SfaGeom& g, float scale, int32_t* status,
                                       cudaStream_t st) {
   using namespace tcbwd256;
   Params p;
   const SfaGeom gq = query_geom(g);
-  if (!make_rows_tmap(&p.tm_q, q, gq, g.Hq, DH, BQ) || !make_rows_tmap(&p.tm_do, dout, gq, g.Hq, DH, BQ) ||
-      !make_rows_tmap(&p.tm_k, k, g, g.Hkv, DH, BK) || !make_rows_tmap(&p.tm_v, v, g, g.Hkv, DH, BK) ||
-      !make_rows_tmap(&p.tm_dq, dq_ws, gq, g.Hq, DH, 16, 4, 32, false))
+  if (!make_rows_tmap(&p.tm_q, q, gq, g.Hq, DH, PR) || !make_rows_tmap(&p.tm_do, dout, gq, g.Hq, DH, PR) ||
+      !make_rows_tmap(&p.tm_k, k, g, g.Hkv, DH, PR) || !make_rows_tmap(&p.tm_v, v, g, g.Hkv, DH, PR))
     return cudaErrorInvalidValue;
   p.lse2 = lse2_ws;
   p.delta = delta_ws;
+  p.dq = (bf16*)dq_out;
+  p.dq_acc = dq_ws;
   p.dk = (bf16*)dk;
   p.dv = (bf16*)dv;
-  p.hchunks = bwd_head_chunks(g, DH);
+  const long long slice = (long long)g.B * g.q_ns * g.Lv * g.Hkv * DH;  // elements of dV (or dK) of one chunk
+  const int ws_chunks = bwd_head_chunks(g, DH);
+  long long room = ws_chunks > 1 ? ws_chunks : 0;
   p.dkv = dkv_ws;
+  const long long acc_room = dq_out ? (long long)g.B * g.q_nL * g.Hq * DH / (2 * slice) : 0;
+  if (acc_room > room) {
+    room = acc_room;
+    p.dkv = dq_ws;
+  }
+  p.head_pairs = (g.Hq / g.Hkv) % 2 == 0;
+  const int rows = p.head_pairs ? BM : 2 * BM, nh = p.head_pairs ? g.Hq / 2 : g.Hq;
+  const long long ndq = (long long)((g.Lq + rows - 1) / rows) * nh * g.q_ns * g.B;
+  p.hchunks = head_chunks(g, room, ndq);
+  if (p.hchunks > 1 && p.dkv == nullptr) return cudaErrorInvalidValue;
   p.g = g;
   p.scale = scale;
   p.scale_log2 = scale * 1.4426950408889634f;
   p.status = status;
-  const size_t nkv = bwd_dkv_slice(g, DH);
-  if (p.hchunks > 1 && dkv_ws == nullptr) return cudaErrorInvalidValue;
-  const int smem = kSmemBytes;
-  auto kern = g.window > 0 ? bwd256_kernel<true> : bwd256_kernel<false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  p.nkv = (int)(key_items(g) * p.hchunks);
+  const long long grid = 2 * (2LL * p.nkv + ndq);
+  cudaError_t e = cudaFuncSetAttribute(bwd256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)((g.Lv + BK - 1) / BK) * (unsigned)(2 * p.hchunks * g.Hkv * g.q_ns * g.B);
-  kern<<<grid, NTHREADS, smem, st>>>(p);
+  bwd256_kernel<<<(unsigned)grid, NTHREADS, kSmemBytes, st>>>(p);
   e = cudaGetLastError();
   if (e != cudaSuccess || p.hchunks == 1) return e;
-  const long long n8 = (long long)nkv / 8;
-  dkv_finalize_kernel<<<(unsigned)((n8 + 255) / 256), 256, 0, st>>>(dkv_ws, (bf16*)dk, (bf16*)dv, g, p.hchunks);
+  const long long n8 = slice / 8;
+  dkv_finalize_kernel<<<(unsigned)((n8 + 255) / 256), 256, 0, st>>>(p.dkv, (bf16*)dk, (bf16*)dv, g, p.hchunks);
   return cudaGetLastError();
 }
 
