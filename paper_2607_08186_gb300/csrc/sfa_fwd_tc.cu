@@ -15,17 +15,38 @@
 // one head (the second tile then runs one key tile longer: measured as about 2 us of
 // a WITHIN CTA's 35 us, the first tile's softmax warps idle meanwhile).
 // Roles (320 threads):
-//   warp 0      TMA producer: both Q tiles once, then K/V tiles into a 2-stage ring;
-//               owns TMEM.
+//   warp 0      TMA producer: both Q tiles once, then the tiles K(lo), V(lo), K(lo+1),
+//               V(lo+1), ... into a ring of single K or V tiles.
 //   warp 1      MMA issuer: the whole warp runs the issue loop, one elected lane
-//               issues.  Per key tile and group: S_g = Q_g K^T (SS) into the group's
-//               128 TMEM columns, O_g += P_g V (TS: P_g read from TMEM) into its O
+//               issues; owns TMEM.  Per key tile and group: S_g = Q_g K^T (SS) into the
+//               group's 128 TMEM columns, O_g += P_g V (TS: P_g read from TMEM) into its O
 //               columns; the next S_g is issued after the PV that reads P_g.
 //   warps 2..5, 6..9  softmax of group 0 / 1: one thread per query row (its TMEM
 //               lane); online softmax in fp32 with exp2 (packed f32x2 arithmetic),
-//               P packed to bf16 over the first 64 columns of S_g, O_g rescaled in
-//               TMEM only when the running max grows by more than 2^8, epilogue.
+//               P packed to bf16 over the first 64 columns of S_g and released to the PV
+//               in two halves, O_g rescaled in TMEM only when the running max grows by
+//               more than 2^8, epilogue.
 // K/V tiles use the 128-byte swizzle written by TMA.  Every mbarrier wait is bounded.
+//
+// What bounds it: a group's own chain P -> PV -> next S -> softmax: 1024 cycles of MMAs,
+// about 300 of signals and 1300 of softmax (of those 600 are the SFU's 128 exp2 per row),
+// under which the other group's 1024 cycles of MMAs run: about 2550 per key tile and group
+// pair, against 2048 of MMAs.  A tensor pipe that waits costs most: the issuer holds
+// about five MMAs (360 cycles) in its queue, a wait on a completed barrier takes 90
+// cycles, 215 right after a commit, and a second commit 110, since barriers live in the
+// shared memory that the S MMAs read at its full rate.  So between the last MMA of a batch
+// and the first of the next the issuer only commits once and waits once (for P); a
+// softmax warp, idle then, has waited for the K / V tiles, and ring slots are released
+// where no wait follows.  K and V tiles have slots of their own, so K(j+1) is on its way
+// while V(j) is in use (a two-stage ring of K and V together left S(j+1) waiting for its
+// load, 3450 cycles per tile).
+// Measured: 470 -> 375 us for an intra-stream layer (B=1, L=4096, n=4, 32 over 8 heads of
+// dim 128), 6.26 -> 5.27 ms for a cross-stream one of 32768 positions (1.67 PFLOP/s), 110
+// -> 93 us at head dim 64 (B=4, L=1501, n=3, 16 over 4 heads).  A CTA's fixed part, about
+// 8500 cycles, is what separates the intra-stream layer from the tile time.
+// Slower: one issuer per group (459 us: the groups' MMAs interleave and their softmaxes
+// meet on the SFU), the tile waits inside the S batch (440 us) or between the halves of P
+// (454 us), two single-tile CTAs per SM (463 us: K and V are loaded twice).
 #include "tc_common.cuh"
 
 namespace hdsfa {
@@ -33,7 +54,7 @@ namespace hdsfa {
 typedef __nv_bfloat16 bf16;
 
 namespace tcfwd {
-constexpr int BM = 128, BN = 128, NST = 2, NG = 2, NTHREADS = 64 + NG * 128;
+constexpr int BM = 128, BN = 128, NG = 2, NTHREADS = 64 + NG * 128;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleThreshold = 8.0f;  // log2 units: P stays <= 256 between O rescales
@@ -41,12 +62,16 @@ constexpr float kRescaleThreshold = 8.0f;  // log2 units: P stays <= 256 between
 template <int DH>
 struct Smem {
   bf16 q[NG][BM * DH];  // per query tile: DH/64 swizzle blocks of [BM][64]
-  bf16 k[NST][BN * DH];
-  bf16 v[NST][BN * DH];
-  uint64_t q_full, kv_full[NST], kv_empty[NST], s_full[NG], p_full[NG], o_done[NG], drain;
+  static constexpr int NSLOT = DH == 64 ? 10 : 5;
+  bf16 ring[NSLOT][BN * DH];  // one K or V tile each
+  uint64_t q_full[NG], full[NSLOT], empty[NSLOT], s_full[NG], p_full[NG][2], o_done[NG], drain;
   uint32_t tmem_base;
   int abort;
 };
+// The layout needs 1024-byte alignment; the kernel checks the actual pad on entry.
+template <int DH>
+constexpr int smem_bytes() { return (int)sizeof(Smem<DH>) + 1024 < 232448 ? (int)sizeof(Smem<DH>) + 1024 : 232448; }
+static_assert(sizeof(Smem<128>) <= 232448, "forward shared memory exceeds 227 KB");
 
 struct Params {
   CUtensorMap tm_q, tm_k, tm_v;
@@ -57,11 +82,6 @@ struct Params {
   int32_t* status;
   int head_pairs;  // 1: a CTA's two query tiles are the same rows of two heads of one K/V group
 };
-
-// Key row c visible from the query at key row rq (= r*qstep + qoff).
-HD_DEVINLINE bool visible(int rq, int c, int Lv, int window) {
-  return c <= rq && c < Lv && (window <= 0 || rq - c < window);
-}
 
 // Key-tile range [lo, hi] of the query tile starting at row m0 (hi < lo: no rows).
 HD_DEVINLINE void tile_range(const SfaGeom& G, int m0, int& lo, int& hi) {
@@ -81,7 +101,17 @@ HD_DEVINLINE void tile_range(const SfaGeom& G, int m0, int& lo, int& hi) {
 // modes' softmax carries none of that code.
 template <int DH, bool NAIVE>
 __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant__ Params P) {
+  constexpr int NSLOT = Smem<DH>::NSLOT;
   extern __shared__ uint8_t smem_raw[];
+  {
+    uint32_t dyn;
+    asm("mov.u32 %0, %%dynamic_smem_size;\n" : "=r"(dyn));
+    const uintptr_t base = reinterpret_cast<uintptr_t>(smem_raw);
+    if (((base + 1023) & ~uintptr_t(1023)) - base + sizeof(Smem<DH>) > dyn) {  // uniform: nothing touched yet
+      if (threadIdx.x == 0) set_status(P.status, HD_DEVBIT_TIMEOUT);
+      return;
+    }
+  }
   Smem<DH>& sm = *reinterpret_cast<Smem<DH>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const SfaGeom& G = P.g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -116,21 +146,22 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
   for (int g = 1; g < NG; ++g) n_hi = max(n_hi, hi[g]);
 
   if (threadIdx.x == 0) {
-    mbar_init(&sm.q_full, 1);
-    for (int i = 0; i < NST; ++i) {
-      mbar_init(&sm.kv_full[i], 1);
-      mbar_init(&sm.kv_empty[i], 1);
+    for (int i = 0; i < NSLOT; ++i) {
+      mbar_init(&sm.full[i], 1);
+      mbar_init(&sm.empty[i], 1);
     }
     for (int g = 0; g < NG; ++g) {
+      mbar_init(&sm.q_full[g], 1);
       mbar_init(&sm.s_full[g], 1);
-      mbar_init(&sm.p_full[g], 128);
+      mbar_init(&sm.p_full[g][0], 4);  // one arrival per softmax warp of the group
+      mbar_init(&sm.p_full[g][1], 4);
       mbar_init(&sm.o_done[g], 1);
     }
     mbar_init(&sm.drain, 1);
     sm.abort = 0;
     fence_mbar_init();
   }
-  if (warp == 0) {
+  if (warp == 1) {
     tmem_alloc(&sm.tmem_base, 512);
     tmem_relinquish();
   }
@@ -143,94 +174,112 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      tma_prefetch(&P.tm_q);
-      tma_prefetch(&P.tm_k);
-      tma_prefetch(&P.tm_v);
-      mbar_arrive_expect_tx(&sm.q_full, NG * BM * DH * 2);
-      for (int g = 0; g < NG; ++g)
-        for (int c = 0; c < DH / 64; ++c)
-          tma_load_5d(sm.q[g] + c * BM * 64, &P.tm_q, &sm.q_full, c * 64, hd[g], s, qm[g], b);
-      int issued = 0;
-      for (int j = n_lo; j <= n_hi; ++j, ++issued) {
-        const int it = j - n_lo, st = it % NST;
-        if (it >= NST && !mbar_wait(&sm.kv_empty[st], ((it / NST) - 1) & 1, abort, P.status)) break;
-        mbar_arrive_expect_tx(&sm.kv_full[st], 2 * BN * DH * 2);
-        for (int c = 0; c < DH / 64; ++c) {
-          tma_load_5d(sm.k[st] + c * BN * 64, &P.tm_k, &sm.kv_full[st], c * 64, kvh, sk, j * BN, b);
-          tma_load_5d(sm.v[st] + c * BN * 64, &P.tm_v, &sm.kv_full[st], c * 64, kvh, sk, j * BN, b);
+      int slot = 0, ph = 1, issued = 0;  // empty-barrier phase: the first lap does not wait
+      bool ok = true;
+      auto load_tile = [&](const CUtensorMap* tm, int j) {
+        if (!ok || !mbar_wait(&sm.empty[slot], ph, abort, P.status)) {
+          ok = false;
+          return;
         }
+        mbar_arrive_expect_tx(&sm.full[slot], BN * DH * 2);
+        for (int c = 0; c < DH / 64; ++c)
+          tma_load_5d(sm.ring[slot] + c * BN * 64, tm, &sm.full[slot], c * 64, kvh, sk, j * BN, b);
+        ++issued;
+        if (++slot == NSLOT) {
+          slot = 0;
+          ph ^= 1;
+        }
+      };
+      auto load_q = [&](int g) {
+        mbar_arrive_expect_tx(&sm.q_full[g], BM * DH * 2);
+        for (int c = 0; c < DH / 64; ++c)
+          tma_load_5d(sm.q[g] + c * BM * 64, &P.tm_q, &sm.q_full[g], c * 64, hd[g], s, qm[g], b);
+      };
+      load_q(0);
+      if (n_lo <= n_hi) load_tile(&P.tm_k, n_lo);
+      load_q(1);
+      for (int j = n_lo; ok && j <= n_hi; ++j) {
+        load_tile(&P.tm_v, j);
+        if (j < n_hi) load_tile(&P.tm_k, j + 1);
       }
       // every copy this thread started lands before the CTA may exit
-      mbar_drain(&sm.q_full, 0);
-      for (int it = max(0, issued - NST); it < issued; ++it) mbar_drain(&sm.kv_full[it % NST], (it / NST) & 1);
+      for (int g = 0; g < NG; ++g) mbar_drain(&sm.q_full[g], 0);
+      for (int u = max(0, issued - NSLOT); u < issued; ++u) mbar_drain(&sm.full[u % NSLOT], (u / NSLOT) & 1);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     // The whole warp runs the loop (warp-uniform operands); one elected lane issues.
-    {
-      constexpr uint32_t idS = idesc_bf16(BM, BN, 0, 0);  // S[q][kv] = Q K^T (both K-major)
-      constexpr uint32_t idO = idesc_bf16(BM, DH, 0, 1);  // O[q][d] += P V   (P in TMEM, V MN-major)
-      int ps[NG] = {0, 0};                                  // per-group P phases consumed
-      bool ok = __all_sync(0xffffffffu, mbar_wait(&sm.q_full, 0, abort, P.status));
-      int kv_ready = n_lo - 1;                              // highest key tile known loaded
-      auto wait_kv = [&](int j) -> bool {
-        if (j <= kv_ready) return true;
-        const int it = j - n_lo;
-        if (!__all_sync(0xffffffffu, mbar_wait(&sm.kv_full[it % NST], (it / NST) & 1, abort, P.status))) return false;
-        kv_ready = j;
-        tc_fence_after();
-        return true;
-      };
-      // Operand descriptors are encoded once; k-step kk adds its byte offset / 16 to the
-      // 64-bit descriptor (the address field; shared addresses stay below 256 KB), which
-      // keeps the instructions between consecutive MMAs (and so the issue gaps) small.
-      static_assert(BM == 128 && BN == 128 && NST == 2 && NG == 2, "descriptor bases below");
-      const uint64_t qK0 = sdesc_sw128(smem_u32(sm.q[0]), 16, 1024), qK1 = sdesc_sw128(smem_u32(sm.q[1]), 16, 1024);
-      const uint64_t kK0 = sdesc_sw128(smem_u32(sm.k[0]), 16, 1024), kK1 = sdesc_sw128(smem_u32(sm.k[1]), 16, 1024);
-      const uint64_t vM0 = sdesc_sw128(smem_u32(sm.v[0]), BN * 128, 1024),
-                     vM1 = sdesc_sw128(smem_u32(sm.v[1]), BN * 128, 1024);
-      auto issue_s = [&](int g, int j) {
-        const uint64_t qd = g ? qK1 : qK0, kd = ((j - n_lo) & 1) ? kK1 : kK0;
+    constexpr uint32_t idS = idesc_bf16(BM, BN, 0, 0);  // S[q][kv] = Q K^T (both K-major)
+    constexpr uint32_t idO = idesc_bf16(BM, DH, 0, 1);  // O[q][d] += P V   (P in TMEM, V MN-major)
+    static_assert(BM == 128 && BN == 128 && NG == 2, "descriptor offsets below");
+    // Operand descriptors are encoded once; a slot or k-step adds its byte offset / 16 to
+    // the 64-bit descriptor (the address field; shared addresses stay below 256 KB), which
+    // keeps the instructions between consecutive MMAs (and so the issue gaps) small.
+    const uint64_t qd0 = sdesc_sw128(smem_u32(sm.q[0]), 16, 1024);
+    const uint64_t kd0 = sdesc_sw128(smem_u32(sm.ring[0]), 16, 1024);
+    const uint64_t vd0 = sdesc_sw128(smem_u32(sm.ring[0]), BN * 128, 1024);
+    constexpr int TILE16 = BN * DH * 2 / 16;
+    auto wait_w = [&](uint64_t* bar, int par) -> bool {
+      if (!__all_sync(0xffffffffu, mbar_wait(bar, par & 1, abort, P.status))) return false;
+      tc_fence_after();
+      return true;
+    };
+    auto issue_s = [&](int g, int slot) {
+      const uint64_t qd = qd0 + (uint64_t)(g * (BM * DH * 2 / 16)), kd = kd0 + (uint64_t)(slot * TILE16);
 #pragma unroll
-        for (int kk = 0; kk < DH / 16; ++kk) {
-          const uint64_t off = (uint64_t)((kk >> 2) * (128 * 128 / 16) + (kk & 3) * 2);
-          tc_mma_ss_w(tmem + g * 128, qd + off, kd + off, idS, kk > 0 ? 1u : 0u);
-        }
-        tc_commit_w(&sm.s_full[g]);
-      };
-      auto issue_pv = [&](int g, int j) -> bool {
-        if (!__all_sync(0xffffffffu, mbar_wait(&sm.p_full[g], ps[g] & 1, abort, P.status))) return false;
-        ++ps[g];
-        tc_fence_after();
-        const uint64_t vd = ((j - n_lo) & 1) ? vM1 : vM0;
-#pragma unroll
-        for (int kk = 0; kk < BN / 16; ++kk)
-          tc_mma_ts_w(tmem + 256 + g * DH, tmem + g * 128 + kk * 8, vd + (uint64_t)(kk * 16 * 128 / 16), idO,
-                    (j > lo[g] || kk > 0) ? 1u : 0u);
-        return true;
-      };
-      if (ok && n_hi >= n_lo && wait_kv(n_lo)) {
-        for (int g = 0; g < NG; ++g)
-          if (lo[g] <= n_lo && n_lo <= hi[g]) issue_s(g, n_lo);
-        for (int j = n_lo; ok && j <= n_hi; ++j) {
-          for (int g = 0; ok && g < NG; ++g) {
-            if (lo[g] <= j && j <= hi[g]) {
-              if (!issue_pv(g, j)) { ok = false; break; }
-              if (j == hi[g]) tc_commit_w(&sm.o_done[g]);
-            }
-            // S of the next tile for this group reuses its S/P columns: issued after its PV
-            if (j + 1 <= hi[g] && lo[g] <= j + 1) {
-              if (!wait_kv(j + 1)) { ok = false; break; }
-              issue_s(g, j + 1);
-            }
-          }
-          tc_commit_w(&sm.kv_empty[(j - n_lo) % NST]);
-        }
+      for (int kk = 0; kk < DH / 16; ++kk) {
+        const uint64_t off = (uint64_t)((kk >> 2) * (128 * 128 / 16) + (kk & 3) * 2);
+        tc_mma_ss_w(tmem + g * 128, qd + off, kd + off, idS, kk > 0 ? 1u : 0u);
       }
-      // every MMA issued above completes before TMEM / smem are released
-      tc_commit_w(&sm.drain);
-      mbar_drain(&sm.drain, 0);
+      tc_commit_w(&sm.s_full[g]);
+    };
+    // P arrives in two halves of 64 keys: the first half's k-steps run while the softmax
+    // computes the second.  The softmax publishes P(j) only after V(j) and K(j+1) have
+    // landed, so the issuer waits for nothing else: each of its waits takes 90 cycles, 215
+    // right after a commit, and a commit after another 110, against about 360 cycles of
+    // queued MMAs.  Releases go where no wait follows at once.
+    auto issue_pv = [&](int g, int j, int slot, int k_done) -> bool {
+      const uint64_t vd = vd0 + (uint64_t)(slot * TILE16);
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        if (!wait_w(&sm.p_full[g][hf], j - lo[g])) return false;
+#pragma unroll
+        for (int kk = hf * 4; kk < hf * 4 + 4; ++kk)
+          tc_mma_ts_w(tmem + 256 + g * DH, tmem + g * 128 + kk * 8, vd + (uint64_t)(kk * 16 * 128 / 16), idO,
+                      (j > lo[g] || kk > 0) ? 1u : 0u);
+        if (hf == 0 && k_done >= 0) tc_commit_w(&sm.empty[k_done]);
+      }
+      return true;
+    };
+    auto next_slot = [](int s) { return s + 1 == NSLOT ? 0 : s + 1; };
+    bool ok = true;
+    int k_done = -1, v_slot = 1;  // K(j), not yet released; V(j) (K(n_lo) is in slot 0)
+    if (n_hi >= n_lo) {
+      ok = wait_w(&sm.full[0], 0);
+      for (int g = 0; ok && g < NG; ++g) {
+        ok = wait_w(&sm.q_full[g], 0);
+        if (ok && lo[g] <= n_lo && n_lo <= hi[g]) issue_s(g, 0);
+      }
+      k_done = 0;
     }
+    for (int j = n_lo; ok && j <= n_hi; ++j) {
+      const int k_slot = next_slot(v_slot);  // K(j+1)
+      for (int g = 0; ok && g < NG; ++g) {
+        if (lo[g] <= j && j <= hi[g]) {
+          if (!issue_pv(g, j, v_slot, k_done)) { ok = false; break; }
+          k_done = -1;
+          if (j == hi[g]) tc_commit_w(&sm.o_done[g]);
+        }
+        if (g == NG - 1) tc_commit_w(&sm.empty[v_slot]);
+        // S of the next tile for this group reuses its S/P columns: issued after its PV
+        if (j + 1 <= hi[g] && lo[g] <= j + 1) issue_s(g, k_slot);
+      }
+      k_done = k_slot;
+      v_slot = next_slot(k_slot);
+    }
+    // every MMA issued above completes before TMEM / smem are released
+    tc_commit_w(&sm.drain);
+    mbar_drain(&sm.drain, 0);
   } else {
     // ------------------------------------------------------------ softmax / epilogue
     const int g = (warp - 2) >> 2;
@@ -249,6 +298,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
     bool ok = true;
     for (int j = lo[g]; j <= hi[g]; ++j) {
       const int i = j - lo[g];
+      // this thread's arrivals on p_full also say that V(j) and K(j+1) have landed (waited
+      // for here, where the softmax waits for S anyway)
+      if (warp == 2 + 4 * g && lane == 0) {
+        const int u = 2 * (j - n_lo) + 1;  // V(j)'s place in the ring's order
+        mbar_wait(&sm.full[u % NSLOT], (u / NSLOT) & 1, abort, P.status);
+        if (j < n_hi) mbar_wait(&sm.full[(u + 1) % NSLOT], ((u + 1) / NSLOT) & 1, abort, P.status);
+      }
+      __syncwarp();
       // tcgen05.ld/st are warp-collective: every wait result is made warp-uniform
       if (!__all_sync(0xffffffffu, mbar_wait(&sm.s_full[g], i & 1, abort, P.status))) {
         ok = false;
@@ -274,9 +331,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
           k = k == 0 ? G.smod - 1 : k - 1;
         }
       } else if (need_mask) {
+        // keys past the query's own row or the end, and (LOCAL) at or below its window edge
+        const int e_hi = min(rq, G.Lv - 1) - j * BN;
 #pragma unroll
         for (int e = 0; e < BN; ++e)
-          if (!visible(rq, j * BN + e, G.Lv, G.window)) x[e] = -INFINITY;
+          if (e > e_hi) x[e] = -INFINITY;
+        if (G.window > 0) {
+          const int e_lo = rq - G.window + 1 - j * BN;
+#pragma unroll
+          for (int e = 0; e < BN; ++e)
+            if (e < e_lo) x[e] = -INFINITY;
+        }
       }
       float mx[8];
 #pragma unroll
@@ -290,45 +355,48 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
       const float m_use = rescale ? m_new : m_run;
       const float neg = (m_use == -INFINITY) ? 0.f : -m_use * c2;
       const uint64_t c2x2 = f2pack(c2, c2), neg2 = f2pack(neg, neg);
+      // P (bf16 pairs) over the first 64 columns of this group's S, published in halves
       uint64_t sum2[4] = {0, 0, 0, 0};
-      uint32_t pk[BN / 2];
-#pragma unroll
-      for (int e = 0; e < BN; e += 2) {
-        float a0, a1;
-        f2unpack(ffma2(f2pack(x[e], x[e + 1]), c2x2, neg2), a0, a1);
-        const float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
-        sum2[(e >> 1) & 3] = fadd2(sum2[(e >> 1) & 3], f2pack(p0, p1));
-        pk[e >> 1] = cvt_bf16x2(p0, p1);
-      }
-      float s0, s1, s2, s3, s4, s5, s6, s7;
-      f2unpack(sum2[0], s0, s1);
-      f2unpack(sum2[1], s2, s3);
-      f2unpack(sum2[2], s4, s5);
-      f2unpack(sum2[3], s6, s7);
-      const float rsum = ((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7));
-      // O_g already holds every earlier tile's PV (its S of this tile was issued after them)
       const bool mine = rescale && m_run != -INFINITY && i > 0;
-      if (__any_sync(0xffffffffu, mine)) {
-        const float alpha = mine ? ex2_approx((m_run - m_use) * c2) : 1.f;
-        l_run *= alpha;
 #pragma unroll
-        for (int c = 0; c < DH / 32; ++c) {
-          uint32_t o[32];
-          tmem_ld32(tO + c * 32, o);
-          tmem_ld_wait();
+      for (int c = 0; c < BN / 32; ++c) {
+        uint32_t pk[16];
 #pragma unroll
-          for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-          tmem_st32(tO + c * 32, o);
+        for (int e = c * 32; e < c * 32 + 32; e += 2) {
+          float a0, a1;
+          f2unpack(ffma2(f2pack(x[e], x[e + 1]), c2x2, neg2), a0, a1);
+          const float p0 = ex2_approx(a0), p1 = ex2_approx(a1);
+          sum2[(e >> 1) & 3] = fadd2(sum2[(e >> 1) & 3], f2pack(p0, p1));
+          pk[(e >> 1) & 15] = cvt_bf16x2(p0, p1);
+        }
+        tmem_st16(tS + c * 16, pk);
+        if (c & 1) {
+          if (c == 1 && __any_sync(0xffffffffu, mine)) {
+            // O_g already holds every earlier tile's PV (its S of this tile was issued after
+            // them).  Looked at here, so that the vote does not delay the exponentials.
+            const float alpha = mine ? ex2_approx((m_run - m_use) * c2) : 1.f;
+            l_run *= alpha;
+#pragma unroll
+            for (int d = 0; d < DH / 16; ++d) {
+              uint32_t o[16];
+              tmem_ld16(tO + d * 16, o);
+              tmem_ld_wait();
+#pragma unroll
+              for (int k = 0; k < 16; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * alpha);
+              tmem_st16(tO + d * 16, o);
+            }
+          }
+          tmem_st_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sm.p_full[g][c >> 1]);
         }
       }
+      float s0, s1, s2, s3;
+      f2unpack(fadd2(sum2[0], sum2[1]), s0, s1);
+      f2unpack(fadd2(sum2[2], sum2[3]), s2, s3);
+      l_run += (s0 + s1) + (s2 + s3);
       m_run = m_use;
-      l_run += rsum;
-      // P (bf16 pairs) over the first 64 columns of this group's S
-#pragma unroll
-      for (int c = 0; c < BN / 32; ++c) tmem_st16(tS + c * 16, pk + c * 16);
-      tmem_st_wait();
-      tc_fence_before();
-      mbar_arrive(&sm.p_full[g]);
     }
     if (ok && hi[g] >= lo[g] && __all_sync(0xffffffffu, mbar_wait(&sm.o_done[g], 0, abort, P.status))) {
       tc_fence_after();
@@ -376,7 +444,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (warp == 1) {
     __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem, 512);
@@ -387,7 +455,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
 // --------------------------------------------------------------------- host
 template <int DH, bool NAIVE>
 static cudaError_t tc_fwd_impl(tcfwd::Params& p, cudaStream_t st) {
-  const int smem = (int)sizeof(tcfwd::Smem<DH>) + 1024;
+  constexpr int smem = tcfwd::smem_bytes<DH>();
   cudaError_t e =
       cudaFuncSetAttribute(tcfwd::fwd_kernel<DH, NAIVE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
