@@ -172,10 +172,11 @@ hd_status_t sfa_bwd(const void* q, const void* k, const void* v, const void* o, 
  * can overlap or time them separately.  Same sizes, mode and workspace as sfa_bwd.
  *   sfa_bwd_prep     : delta = rowsum(dO * O) and lse * log2(e) into the workspace
  *                      (fp32, stream-major), and zero its fp32 dQ accumulator.
- *   sfa_bwd_main     : recompute P on visible pairs, add every dQ contribution
- *                      into the accumulator (at Dh = 256: store the finished sums
- *                      there) and write dk, dv (overwritten).
+ *   sfa_bwd_main     : recompute P on visible pairs, store the finished fp32 sums of
+ *                      dQ into the accumulator and write dk, dv (overwritten).
  *   sfa_bwd_finalize : dq = bf16(scale * accumulator).
+ * (sfa_bwd itself runs the row terms and the main pass only: its dq is written as bf16
+ * by the main pass, from the same sums.)
  * A later phase reads what the earlier one left in the workspace.
  * sfa_bwd_prep is itself the two halves below, for a caller that overlaps them:
  *   sfa_bwd_row_terms: the delta and lse terms only (needs o, so after sfa_fwd);

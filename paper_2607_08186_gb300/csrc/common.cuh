@@ -55,23 +55,21 @@ __host__ __device__ inline SfaGeom query_geom(const SfaGeom& g) {
 constexpr int kRowTermAlign = 128;
 __host__ __device__ inline int row_terms_pitch(int Lv) { return (Lv + kRowTermAlign - 1) / kRowTermAlign * kRowTermAlign; }
 
-// Head chunks of the tensor-core backward.  Its grid is one CTA (two at head dim 256)
-// per 128-row key tile and (b, K/V head, stream); when that leaves SMs idle (short or
-// final-stream problems with few K/V heads), each CTA takes only a chunk of the group's
-// query heads, for up to about four CTAs per SM.  (With one to two CTAs per SM, as in the n = 1
-// and the final-stream intra-stream layers with 8 K/V heads, the partial sums' extra
-// traffic cost more than the better balance gained: 3 % slower.)  Chunk hc writes its dK / dV partial sums (fp32,
-// dK already scaled) to its own slice of a workspace [chunks][2][B][q_ns][Lv][Hkv][Dh]
-// (dV, then dK), and a finalize pass adds the slices in chunk order: the same result,
-// bit for bit, on every run.  This rule sizes the workspace at every head dim; the
-// head-dim-256 kernel has another grid and chooses its own chunk count (head_chunks in
-// sfa_bwd_tc256.cu) within that space.
+// Space for head chunks of the tensor-core backward in its workspace.  When there are few
+// (key tile, K/V head, stream) items (short or final-stream problems with few K/V heads),
+// each item takes only a chunk of the group's query heads and writes its dK / dV partial
+// sums (fp32, dK already scaled) to its own slice [chunks][2][B][q_ns][Lv][Hkv][Dh] (dV,
+// then dK); a finalize pass adds the slices in chunk order: the same result, bit for bit, on
+// every run.  This rule sizes the workspace (a part of the interface: callers and
+// sfa_bwd_noalloc's limit depend on it); the kernels choose their chunk count within it, or
+// within the space of the fp32 dQ where a call does not use that (head_chunks in
+// sfa_bwd_tc.cu and sfa_bwd_tc256.cu).
 constexpr int kSmCount = 152;
 __host__ __device__ inline int bwd_head_chunks(const SfaGeom& g, int Dh) {
   const long long ctas = (long long)((g.Lv + 127) / 128) * (Dh == 256 ? 2 : 1) * g.Hkv * g.q_ns * g.B;
   const int grp = g.Hq / g.Hkv;
   if (ctas >= kSmCount || grp < 2) return 1;
-  long long want = (4 * kSmCount + ctas - 1) / ctas;  // 2 or 6 per SM: 3.5 % / 1 % slower
+  long long want = (4 * kSmCount + ctas - 1) / ctas;
   const int hs = (int)(want < grp ? want : grp);
   const int per = (grp + hs - 1) / hs;
   return (grp + per - 1) / per;
@@ -79,6 +77,23 @@ __host__ __device__ inline int bwd_head_chunks(const SfaGeom& g, int Dh) {
 // Elements of one slice half (dV or dK of one chunk); 0 without chunks.
 __host__ __device__ inline size_t bwd_dkv_slice(const SfaGeom& g, int Dh) {
   return bwd_head_chunks(g, Dh) > 1 ? (size_t)g.B * g.q_ns * g.Lv * g.Hkv * Dh : 0;
+}
+
+// Division of 0 <= n < 2^31 by a launch constant d >= 1 as a multiplication: with
+// s = ceil(log2 d) and m = ceil(2^(31+s) / d) < 2^32, m d exceeds 2^(31+s) by less than d <=
+// 2^s, so n m / 2^(31+s) exceeds n / d by less than 2^-s <= 1 / d and has its integer part.
+// (A tensor-core CTA's index arithmetic, a chain of divisions, took 1150 to 1580 cycles.)
+struct FastDiv {
+  uint32_t m;
+  int sh;
+};
+inline FastDiv make_fast_div(uint32_t d) {
+  int s = 0;
+  while ((1ull << s) < d) ++s;
+  return FastDiv{(uint32_t)(((1ull << (31 + s)) + d - 1) / d), 31 + s};
+}
+__host__ __device__ inline int fast_div(int n, const FastDiv& f) {
+  return (int)(((unsigned long long)(uint32_t)n * f.m) >> f.sh);
 }
 
 HD_DEVINLINE uint32_t smem_u32(const void* p) {

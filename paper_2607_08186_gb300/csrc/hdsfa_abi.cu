@@ -32,8 +32,8 @@ cudaError_t launch_sfa_bwd_prep(const void* o, const void* dout, const float* ls
                                 float* delta_ws, float* dq_ws, const SfaGeom& g, int Dh,
                                 cudaStream_t st, bool zero = true);
 cudaError_t launch_sfa_bwd_clear(float* dq_ws, const SfaGeom& g, int Dh, cudaStream_t st);
-cudaError_t launch_sfa_bwd_main_tc(const void* q, const void* k, const void* v, const void* dout, void* dk,
-                                   void* dv, const float* lse2_ws, const float* delta_ws, float* dq_ws,
+cudaError_t launch_sfa_bwd_main_tc(const void* q, const void* k, const void* v, const void* dout, void* dq_out,
+                                   void* dk, void* dv, const float* lse2_ws, const float* delta_ws, float* dq_ws,
                                    float* dkv_ws, const SfaGeom& g, int Dh, float scale, int32_t* status,
                                    cudaStream_t st);
 cudaError_t launch_sfa_bwd_main_tc256(const void* q, const void* k, const void* v, const void* dout, void* dq_out,
@@ -303,12 +303,12 @@ hd_status_t sfa_bwd_main(const void* q, const void* k, const void* v, const void
   BwdWs ws;
   if ((st = split_ws(g, Dh, workspace, workspace_bytes, &ws)) != HD_OK) return st;
   const float scale = resolve_scale(softmax_scale, Dh);
-  // tcgen05 kernels at every head dim (at 256 the accumulator is stored, not added to)
+  // the fp32 sums of dQ go to the workspace's accumulator (sfa_bwd takes them as bf16)
   if (Dh == 256)
     return cuda_status(hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, nullptr, dk, dv, ws.lse2, ws.delta, ws.dq,
                                                         ws.dkv, g, scale, dev_status, stream));
-  return cuda_status(hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, Dh,
-                                                   scale, dev_status, stream));
+  return cuda_status(hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, nullptr, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv,
+                                                   g, Dh, scale, dev_status, stream));
 }
 
 hd_status_t sfa_bwd_finalize(void* dq, int B, int L, int n, int Hq, int Hkv, int Dh,
@@ -339,21 +339,15 @@ hd_status_t sfa_bwd(const void* q, const void* k, const void* v, const void* o, 
   if (st != HD_OK) return st;
   BwdWs ws;
   if ((st = split_ws(g, Dh, workspace, workspace_bytes, &ws)) != HD_OK) return st;
-  if (Dh == 256) {  // dQ leaves the main pass as bf16: no accumulator to clear or convert
-    const float scale = resolve_scale(softmax_scale, Dh);
-    cudaError_t e = hdsfa::launch_sfa_bwd_prep(o, dout, lse, ws.lse2, ws.delta, ws.dq, query_geom(g), Dh, stream, false);
-    if (e == cudaSuccess)
-      e = hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, scale,
-                                           dev_status, stream);
-    return cuda_status(e);
-  }
-  st = sfa_bwd_prep(o, dout, lse, B, L, n, Hq, Hkv, Dh, mode, workspace, workspace_bytes, stream);
-  if (st != HD_OK) return st;
-  st = sfa_bwd_main(q, k, v, dout, dk, dv, B, L, n, Hq, Hkv, Dh, softmax_scale, mode, window, workspace,
-                    workspace_bytes, dev_status, stream);
-  if (st != HD_OK) return st;
-  return sfa_bwd_finalize(dq, B, L, n, Hq, Hkv, Dh, softmax_scale, mode, workspace,
-                          workspace_bytes, stream);
+  // dQ leaves the main pass as bf16: no accumulator to clear or convert
+  const float scale = resolve_scale(softmax_scale, Dh);
+  cudaError_t e = hdsfa::launch_sfa_bwd_prep(o, dout, lse, ws.lse2, ws.delta, ws.dq, query_geom(g), Dh, stream, false);
+  if (e == cudaSuccess)
+    e = Dh == 256 ? hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g,
+                                                     scale, dev_status, stream)
+                  : hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, Dh,
+                                                  scale, dev_status, stream);
+  return cuda_status(e);
 }
 
 // Sizes of a decode step: max_tokens bounds every sequence's length and the cache
@@ -441,7 +435,7 @@ hd_status_t sfa_bwd_final(const void* q, const void* k, const void* v, const voi
   if ((st = split_ws(g, Dh, workspace, workspace_bytes, &ws)) != HD_OK) return st;
   const float scale = resolve_scale(softmax_scale, Dh);
   const SfaGeom gq = query_geom(g);
-  cudaError_t e = hdsfa::launch_sfa_bwd_prep(o, dout, lse, ws.lse2, ws.delta, ws.dq, gq, Dh, stream, Dh != 256);
+  cudaError_t e = hdsfa::launch_sfa_bwd_prep(o, dout, lse, ws.lse2, ws.delta, ws.dq, gq, Dh, stream, false);
   if (e == cudaSuccess && mode == SFA_WITHIN) {
     // only stream n-1's keys are seen by the final-stream queries: the other rows are zero
     const size_t bytes = (size_t)B * n * L * Hkv * Dh * 2;
@@ -453,10 +447,9 @@ hd_status_t sfa_bwd_final(const void* q, const void* k, const void* v, const voi
       e = hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, scale,
                                            dev_status, stream);
     else
-      e = hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, Dh, scale, dev_status,
-                                        stream);
+      e = hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, Dh, scale,
+                                        dev_status, stream);
   }
-  if (e == cudaSuccess && Dh != 256) e = hdsfa::launch_sfa_bwd_finalize(dq, ws.dq, gq, Dh, scale, stream);
   return cuda_status(e);
 }
 

@@ -6,8 +6,8 @@
 //           of any stream is contiguous floats (a single bulk copy).  Negated so the
 //           backward folds them in with one add / fused multiply-add.  Rows in
 //           [Lv, Lvp) get -lse2 = -inf and -delta = 0 (their P and dS vanish).
-//           Also zeroes the fp32 dQ accumulator (or leaves that to clear, which needs
-//           nothing from the forward and may run beside it on another stream).
+//           Also zeroes the fp32 dQ accumulator where asked to (sfa_bwd_prep; clear
+//           alone may run on another stream).
 // finalize: dq = bf16(scale * accumulator), round to nearest even.
 #include "common.cuh"
 

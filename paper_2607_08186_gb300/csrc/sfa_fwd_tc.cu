@@ -40,7 +40,7 @@
 // where no wait follows.  K and V tiles have slots of their own, so K(j+1) is on its way
 // while V(j) is in use (a two-stage ring of K and V together left S(j+1) waiting for its
 // load, 3450 cycles per tile).
-// Measured: 470 -> 375 us for an intra-stream layer (B=1, L=4096, n=4, 32 over 8 heads of
+// Measured: 470 -> 372 us for an intra-stream layer (B=1, L=4096, n=4, 32 over 8 heads of
 // dim 128), 6.26 -> 5.27 ms for a cross-stream one of 32768 positions (1.67 PFLOP/s), 110
 // -> 93 us at head dim 64 (B=4, L=1501, n=3, 16 over 4 heads).  A CTA's fixed part, about
 // 8500 cycles, is what separates the intra-stream layer from the tile time.
@@ -81,6 +81,7 @@ struct Params {
   float scale_log2;
   int32_t* status;
   int head_pairs;  // 1: a CTA's two query tiles are the same rows of two heads of one K/V group
+  FastDiv d_rank, d_hns, d_ns, d_grp;
 };
 
 // Key-tile range [lo, hi] of the query tile starting at row m0 (hi < lo: no rows).
@@ -115,36 +116,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
   Smem<DH>& sm = *reinterpret_cast<Smem<DH>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const SfaGeom& G = P.g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // A CTA's two query tiles: with head_pairs the same 128 rows of heads 2x and 2x+1
-  // (one K/V group: both tiles see exactly the same key tiles and finish together),
-  // else rows m0 and m0 + 128 of one head (the second tile sees one more key tile).
-  const int hp = P.head_pairs;
-  const int rows_per_cta = hp ? BM : NG * BM;
-  const int ncta = (G.Lq + rows_per_cta - 1) / rows_per_cta;
-  const int nh = hp ? G.Hq / NG : G.Hq;  // head slots of the grid
-  // linear grid, query-tile rank slowest: the last query tiles (the most key tiles to
-  // visit) of every head, stream and batch launch first
-  const int per_rank = nh * G.q_ns * G.B;
-  const int mt = ncta - 1 - (int)blockIdx.x / per_rank;
-  const int hsb = (int)blockIdx.x % per_rank;
-  const int b = hsb / (nh * G.q_ns), hx = (hsb / G.q_ns) % nh, s = hsb % G.q_ns;
-  int qm[NG], hd[NG];  // first query row and head of each group's tile
-#pragma unroll
-  for (int g = 0; g < NG; ++g) {
-    qm[g] = hp ? mt * BM : mt * NG * BM + g * BM;
-    hd[g] = hp ? NG * hx + g : hx;
-  }
-  const int h = hd[0];
-  const int sk = s + G.kv_s0;  // stream of the key problem
-  const int kvh = h / (G.Hq / G.Hkv);
-  int lo[NG], hi[NG];
-#pragma unroll
-  for (int g = 0; g < NG; ++g) tile_range(G, qm[g], lo[g], hi[g]);
-  const int n_lo = lo[0];
-  int n_hi = hi[0];
-#pragma unroll
-  for (int g = 1; g < NG; ++g) n_hi = max(n_hi, hi[g]);
-
   if (threadIdx.x == 0) {
     for (int i = 0; i < NSLOT; ++i) {
       mbar_init(&sm.full[i], 1);
@@ -164,12 +135,48 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
   if (warp == 1) {
     tmem_alloc(&sm.tmem_base, 512);
     tmem_relinquish();
+    tc_fence_before();
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = sm.tmem_base;
+  // A CTA's two query tiles: with head_pairs the same 128 rows of heads 2x and 2x+1
+  // (one K/V group: both tiles see exactly the same key tiles and finish together),
+  // else rows m0 and m0 + 128 of one head (the second tile sees one more key tile).
+  const int hp = P.head_pairs;
+  const int rows_per_cta = hp ? BM : NG * BM;
+  const int ncta = (G.Lq + rows_per_cta - 1) / rows_per_cta;
+  const int nh = hp ? G.Hq / NG : G.Hq;  // head slots of the grid
+  // linear grid, query-tile rank slowest: the last query tiles (the most key tiles to
+  // visit) of every head, stream and batch launch first
+  const int per_rank = nh * G.q_ns * G.B;
+  const int rank = fast_div((int)blockIdx.x, P.d_rank);
+  const int mt = ncta - 1 - rank, hsb = (int)blockIdx.x - rank * per_rank;
+  const int b = fast_div(hsb, P.d_hns), hs = hsb - b * nh * G.q_ns;
+  const int hx = fast_div(hs, P.d_ns), s = hs - hx * G.q_ns;
+  int qm[NG], hd[NG];  // first query row and head of each group's tile
+#pragma unroll
+  for (int g = 0; g < NG; ++g) {
+    qm[g] = hp ? mt * BM : mt * NG * BM + g * BM;
+    hd[g] = hp ? NG * hx + g : hx;
+  }
+  const int h = hd[0];
+  const int sk = s + G.kv_s0;  // stream of the key problem
+  const int kvh = fast_div(h, P.d_grp);
+  int lo[NG], hi[NG];
+#pragma unroll
+  for (int g = 0; g < NG; ++g) tile_range(G, qm[g], lo[g], hi[g]);
+  const int n_lo = lo[0];
+  int n_hi = hi[0];
+#pragma unroll
+  for (int g = 1; g < NG; ++g) n_hi = max(n_hi, hi[g]);
+
   volatile int* abort = &sm.abort;
+  uint32_t tmem = 0;
+  if (warp == 0) {
+    named_bar_arrive(1, NTHREADS);  // the producer does not wait for the TMEM allocation
+  } else {
+    named_bar_sync(1, NTHREADS);
+    tc_fence_after();
+    tmem = sm.tmem_base;
+  }
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -479,6 +486,11 @@ cudaError_t launch_sfa_fwd_tc(const void* q, const void* k, const void* v, void*
   p.scale_log2 = scale * tcfwd::kLog2e;
   p.status = status;
   p.head_pairs = (g.Hq / g.Hkv) % tcfwd::NG == 0;
+  const int nh = p.head_pairs ? g.Hq / tcfwd::NG : g.Hq;
+  p.d_rank = make_fast_div((uint32_t)(nh * g.q_ns * g.B));
+  p.d_hns = make_fast_div((uint32_t)(nh * g.q_ns));
+  p.d_ns = make_fast_div((uint32_t)g.q_ns);
+  p.d_grp = make_fast_div((uint32_t)(g.Hq / g.Hkv));
   if (Dh == 64) return tc_fwd_impl<64, false>(p, st);
   return g.smod > 1 ? tc_fwd_impl<128, true>(p, st) : tc_fwd_impl<128, false>(p, st);
 }
