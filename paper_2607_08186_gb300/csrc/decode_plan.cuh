@@ -5,7 +5,7 @@
 namespace hdsfa {
 
 struct DecodePlan {
-  int G, M, ngroups, nsplit, chunk, rg;
+  int G, M, ngroups, nsplit, rg;
   bool tc;  // head dim 256 with <= 128 query rows per K/V head: the tcgen05 kernel
   size_t part_o_bytes, part_ml_bytes;
 };

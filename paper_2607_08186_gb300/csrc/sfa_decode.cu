@@ -63,9 +63,10 @@ struct DecodeArgs {
   float* part_o;        // [B][Hkv][ngroups][nsplit][rg][Dh]
   float2* part_ml;      // [B][Hkv][ngroups][nsplit][rg]: (max in log2 units, sum)
   int32_t* status;
-  int B, Lcap, maxT, n, Hq, Hkv, G, M, ngroups, nsplit, chunk, mode, window;
+  int B, Lcap, maxT, n, Hq, Hkv, G, M, ngroups, nsplit, mode, window;
   int rg;               // query rows per row group (the partials' row pitch)
   float scale_log2;
+  FastDiv d_nsplit;
 };
 
 // Programmatic dependent launch: both kernels are launched so that they may start
@@ -81,6 +82,23 @@ HD_DEVINLINE void grid_dep_launch() { asm volatile("griddepcontrol.launch_depend
 HD_DEVINLINE void seq_range(const DecodeArgs& a, int T, int& lo, int& hi) {
   hi = T * a.n;
   lo = a.mode == SFA_LOCAL ? max(0, (T - 1) * a.n - a.window + 1) : 0;
+}
+
+// Positions [k0, k1) of split c of a sequence of T tokens, in whole tiles of `kt`
+// positions: the sequence's own range over all nsplit splits, not a share of max_tokens, so
+// that a batch of different lengths keeps every CTA busy (16 sequences of 8k to 32k tokens,
+// cross-stream: 815 -> 779 us).  Empty for lengths outside [1, max_tokens] and for splits
+// past the range.  (32-bit with a multiplication for the division: in 64 bits this cost a
+// 30 us step 3 us.)
+HD_DEVINLINE void split_range(const DecodeArgs& a, int T, int c, int kt, int& k0, int& k1) {
+  k0 = k1 = 0;
+  if (T < 1 || T > a.maxT) return;
+  int lo, hi;
+  seq_range(a, T, lo, hi);
+  const int tiles = (hi - lo + kt - 1) / kt, per = fast_div(tiles + a.nsplit - 1, a.d_nsplit);
+  if ((long long)c * per >= tiles) return;
+  k0 = lo + c * per * kt;
+  k1 = min(k0 + per * kt, hi);
 }
 
 template <int DH, int MT>
@@ -100,13 +118,8 @@ __global__ void __launch_bounds__(NT) decode_kernel(DecodeArgs a) {
   grid_dep_wait();
   grid_dep_launch();
   const int T = a.lens[b];
-  int k0 = 0, k1 = 0;
-  if (T >= 1 && T <= a.maxT) {
-    int lo, hi;
-    seq_range(a, T, lo, hi);
-    k0 = lo + c * a.chunk;
-    k1 = min(k0 + a.chunk, hi);
-  }
+  int k0, k1;
+  split_range(a, T, c, KT, k0, k1);
   if (k0 >= k1) {  // nothing of this sequence in this split: an empty partial
     for (int i = tid; i < RG; i += NT) pml[i] = make_float2(-INFINITY, 0.f);
     return;
@@ -273,6 +286,7 @@ __global__ void __launch_bounds__(NT) decode_kernel(DecodeArgs a) {
   // [KW][MT*16][DH]: key group kw's O, its head-dim parts side by side; then the key
   // groups' running max and sum (the DS warps of a key group hold the same ones)
   static_assert((KW * MT * 16 * DH + 2 * KW * MT * 16) * 4 <= 2 * STAGES * KT * DH * 2, "merge fits the ring");
+  static_assert(MT * 16 <= NT, "one thread per row");
   float* sO = reinterpret_cast<float*>(sK);
   float* sM = sO + KW * MT * 16 * DH;  // [KW][MT*16]
   float* sL = sM + KW * MT * 16;       // [KW][MT*16]
@@ -291,93 +305,140 @@ __global__ void __launch_bounds__(NT) decode_kernel(DecodeArgs a) {
 #pragma unroll
     for (int i = 0; i < DC / 8; ++i)
 #pragma unroll
-      for (int e4 = 0; e4 < 4; ++e4) {
-        const int row = mt * 16 + g4 + 8 * (e4 >> 1), col = dw * DC + i * 8 + 2 * t4 + (e4 & 1);
-        sO[(kw * MT * 16 + row) * DH + col] = oacc[mt][i][e4];
+      for (int hf = 0; hf < 2; ++hf) {
+        const int row = mt * 16 + g4 + 8 * hf, col = dw * DC + i * 8 + 2 * t4;
+        *reinterpret_cast<float2*>(sO + (kw * MT * 16 + row) * DH + col) =
+            make_float2(oacc[mt][i][2 * hf], oacc[mt][i][2 * hf + 1]);
       }
   }
   __syncthreads();
-  for (int idx = tid; idx < MT * 16 * DH; idx += NT) {
-    const int row = idx / DH, col = idx % DH;
-    float m = -INFINITY;
+  // one thread per row: its maximum and sum over the key groups, whose weights replace
+  // their maxima
+  if (tid < MT * 16) {
+    float m = -INFINITY, l = 0.f;
 #pragma unroll
-    for (int w = 0; w < KW; ++w) m = fmaxf(m, sM[w * MT * 16 + row]);
-    float o = 0.f, l = 0.f;
-    if (m != -INFINITY) {
+    for (int w = 0; w < KW; ++w) m = fmaxf(m, sM[w * MT * 16 + tid]);
 #pragma unroll
-      for (int w = 0; w < KW; ++w) {
-        const float mw = sM[w * MT * 16 + row];
-        const float f = mw == -INFINITY ? 0.f : exp2f(mw - m);
-        o += f * sO[(w * MT * 16 + row) * DH + col];
-        l += f * sL[w * MT * 16 + row];
-      }
+    for (int w = 0; w < KW; ++w) {
+      const float mw = sM[w * MT * 16 + tid], f = mw == -INFINITY ? 0.f : exp2f(mw - m);
+      l += f * sL[w * MT * 16 + tid];
+      sM[w * MT * 16 + tid] = f;
     }
-    po[row * DH + col] = o;
-    if (col == 0) pml[row] = make_float2(m, l);
+    pml[tid] = make_float2(m, l);
+  }
+  __syncthreads();
+  for (int idx = tid; idx < MT * 16 * (DH / 4); idx += NT) {
+    const int row = idx / (DH / 4), c4 = idx % (DH / 4);
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int w = 0; w < KW; ++w) {
+      const float f = sM[w * MT * 16 + row];
+      const float4 v = *reinterpret_cast<const float4*>(sO + (w * MT * 16 + row) * DH + c4 * 4);
+      o.x += f * v.x;
+      o.y += f * v.y;
+      o.z += f * v.z;
+      o.w += f * v.w;
+    }
+    *reinterpret_cast<float4*>(po + row * DH + c4 * 4) = o;
   }
 }
 
-// CTA (K/V head x row group, sequence, 8-column slice x block of 8 rows); one warp per
-// query row, its lanes over the splits: the row's max and sum by warp reductions, then
-// the slice of O as the weighted sum of the splits' partial slices, written as bf16
-// (round to nearest even); the first slice's CTAs also write the natural-log LSE.
+// CTA per query row (row of the group, K/V head x row group, sequence).  Latency-bound: the
+// partials are a few MB in L2.  Threads are DH/4 column quads x split groups; the first
+// nsplit threads turn the splits' maxima into weights (one value each, reduced over the
+// CTA) while every thread's first partials are on their way, the split groups' sums meet in
+// shared memory, and the row leaves as bf16 (round to nearest even) with the natural-log
+// LSE.  Partials of empty splits are not read into the sum.  (One warp per row and 8
+// columns, its lanes over the splits 1 KB and more apart, took 10.5 us for 19 splits of 384
+// rows of 256 columns and 6.5 us for 37 of 128 rows of 128; this 5.2 and 4.3.)
 template <int DH>
 __global__ void __launch_bounds__(256) combine_kernel(DecodeArgs a) {
-  const int g = blockIdx.x / a.ngroups, rg = blockIdx.x % a.ngroups, b = blockIdx.y;
-  const int c8 = blockIdx.z % (DH / 8), rb = blockIdx.z / (DH / 8);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rows = min(a.rg, a.M - rg * a.rg);
+  constexpr int LW = DH / 4, SG = 256 / LW, NB = 8;  // column quads, split groups, loads in flight
+  static_assert(kMaxSplit <= 256, "one thread per split");
+  __shared__ float wgt[kMaxSplit];
+  __shared__ float red[2][8];
+  __shared__ float4 part[SG][LW];
+  const int row = blockIdx.x, g = blockIdx.y / a.ngroups, rg = blockIdx.y % a.ngroups, b = blockIdx.z;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, l4 = tid % LW, sg = tid / LW;
   const size_t pidx0 = (((size_t)b * a.Hkv + g) * a.ngroups + rg) * a.nsplit;
+  const float* po = a.part_o + (pidx0 * a.rg + row) * DH + l4 * 4;
+  const size_t pitch = (size_t)a.rg * DH;  // between a row's partials
   grid_dep_wait();  // every partial of the decode kernel is written
+  const int r = rg * a.rg + row;
   const int T = a.lens[b];
   const bool valid = T >= 1 && T <= a.maxT;
-  if (!valid && blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.x == 0) set_status(a.status, HD_DEVBIT_INDEX);
-  const int row = rb * 8 + warp;
-  if (row < rows) {
-    float m = -INFINITY;
-    for (int c = lane; c < a.nsplit; c += 32) m = fmaxf(m, a.part_ml[(pidx0 + c) * a.rg + row].x);
+  if (!valid && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) set_status(a.status, HD_DEVBIT_INDEX);
+  if (r >= a.M) return;  // the last row group may be short
+  const float2 ml = tid < a.nsplit ? a.part_ml[(pidx0 + tid) * a.rg + row] : make_float2(-INFINITY, 0.f);
+  float4 x[NB];
 #pragma unroll
-    for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    float l = 0.f, acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int c = lane; c < a.nsplit; c += 32) {
-      const float2 ml = a.part_ml[(pidx0 + c) * a.rg + row];
-      const float f = (ml.x == -INFINITY || m == -INFINITY) ? 0.f : exp2f(ml.x - m);
-      l += f * ml.y;
-      if (f != 0.f) {
-        const float4* src = reinterpret_cast<const float4*>(a.part_o + ((pidx0 + c) * a.rg + row) * DH + c8 * 8);
-        const float4 x0 = src[0], x1 = src[1];
-        acc[0] += f * x0.x;
-        acc[1] += f * x0.y;
-        acc[2] += f * x0.z;
-        acc[3] += f * x0.w;
-        acc[4] += f * x1.x;
-        acc[5] += f * x1.y;
-        acc[6] += f * x1.z;
-        acc[7] += f * x1.w;
-      }
-    }
+  for (int k = 0; k < NB; ++k) {
+    const int c = sg + k * SG;
+    if (c < a.nsplit) x[k] = *reinterpret_cast<const float4*>(po + c * pitch);
+  }
+  float m = ml.x;
 #pragma unroll
-    for (int off = 16; off; off >>= 1) {
-      l += __shfl_xor_sync(0xffffffffu, l, off);
+  for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+  if (lane == 0) red[0][warp] = m;
+  __syncthreads();
 #pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], off);
+  for (int w = 0; w < 8; ++w) m = fmaxf(m, red[0][w]);
+  const float f = ml.x == -INFINITY ? 0.f : exp2f(ml.x - m);
+  if (tid < a.nsplit) wgt[tid] = f;
+  float l = f * ml.y;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+  if (lane == 0) red[1][warp] = l;
+  __syncthreads();
+  l = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) l += red[1][w];
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto add = [&](int c, const float4& v) {
+    const float fc = wgt[c];
+    if (fc != 0.f) {
+      acc.x += fc * v.x;
+      acc.y += fc * v.y;
+      acc.z += fc * v.z;
+      acc.w += fc * v.w;
     }
-    if (lane == 0) {
-      const bool ok = valid && l > 0.f;
-      const float inv = ok ? 1.f / l : 0.f;
-      const int r = rg * a.rg + row, s = r / a.G, h = g * a.G + r % a.G;
-      uint4 out;
-      out.x = pack_bf16(acc[0] * inv, acc[1] * inv);
-      out.y = pack_bf16(acc[2] * inv, acc[3] * inv);
-      out.z = pack_bf16(acc[4] * inv, acc[5] * inv);
-      out.w = pack_bf16(acc[6] * inv, acc[7] * inv);
-      *reinterpret_cast<uint4*>(a.o + (((long long)b * a.n + s) * a.Hq + h) * DH + c8 * 8) = out;
-      if (c8 == 0 && a.lse != nullptr)
-        a.lse[((long long)b * a.Hq + h) * a.n + s] = ok ? (m + __log2f(l)) * 0.6931471805599453f : -INFINITY;
+  };
+#pragma unroll
+  for (int k = 0; k < NB; ++k)
+    if (sg + k * SG < a.nsplit) add(sg + k * SG, x[k]);
+  for (int c0 = sg + NB * SG; c0 < a.nsplit; c0 += NB * SG) {
+#pragma unroll
+    for (int k = 0; k < NB; ++k)
+      if (c0 + k * SG < a.nsplit) x[k] = *reinterpret_cast<const float4*>(po + (c0 + k * SG) * pitch);
+#pragma unroll
+    for (int k = 0; k < NB; ++k)
+      if (c0 + k * SG < a.nsplit) add(c0 + k * SG, x[k]);
+  }
+  part[sg][l4] = acc;
+  __syncthreads();
+  if (tid < LW) {
+#pragma unroll
+    for (int k = 1; k < SG; ++k) {
+      const float4 v = part[k][tid];
+      acc.x += v.x;
+      acc.y += v.y;
+      acc.z += v.z;
+      acc.w += v.w;
     }
+    const bool ok = valid && l > 0.f;
+    const float inv = ok ? 1.f / l : 0.f;
+    const int s = r / a.G, h = g * a.G + r % a.G;
+    uint2 out;
+    out.x = pack_bf16(acc.x * inv, acc.y * inv);
+    out.y = pack_bf16(acc.z * inv, acc.w * inv);
+    *reinterpret_cast<uint2*>(a.o + (((long long)b * a.n + s) * a.Hq + h) * DH + tid * 4) = out;
+    if (tid == 0 && a.lse != nullptr)
+      a.lse[((long long)b * a.Hq + h) * a.n + s] = ok ? (m + __log2f(l)) * 0.6931471805599453f : -INFINITY;
   }
 }
 
+// Launched so that it may start under the kernel before it and the decode kernel under it
+// (with the cheaper combine and merge: 36.9 -> 30.6 us per step at batch 1, 8192 tokens).
 // The new token's n K and V rows into the cache at positions (T-1)n + s: one warp per
 // (sequence, stream), 16-byte vectors.  A length outside [1, Lcap] writes nothing and
 // sets HD_DEVBIT_INDEX.
@@ -387,8 +448,10 @@ __global__ void __launch_bounds__(256) append_kernel(const uint4* __restrict__ k
                                                      int row16, int32_t* status) {
   const int lane = threadIdx.x & 31;
   const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  grid_dep_launch();
   if (w >= (long long)B * n) return;
   const int b = (int)(w / n), s = (int)(w % n);
+  grid_dep_wait();  // an earlier step may still read the cache, or write what is read here
   const int T = lens[b];
   if (T < 1 || T > Lcap) {
     if (lane == 0 && s == 0) set_status(status, HD_DEVBIT_INDEX);
@@ -412,10 +475,15 @@ __global__ void __launch_bounds__(256) append_kernel(const uint4* __restrict__ k
 // tiles of the split's cached rows, with the head-dim-256 forward's plan: S in two
 // 128-column TMEM buffers, O in columns 256..511, K / V halves (128 head-dim columns)
 // through a five-slot ring in the issuer's order K(0), then K(j+1), V(j) per tile; warp 0
-// TMA, warp 1 MMA issue, warps 2..5 the online softmax of one row each (per-element mask:
-// position <= the row's own position, its stream in an intra-stream layer, the window in
-// a local one) and the unnormalised partial (O, running max in log2 units, sum) that
-// combine_kernel merges.  Every mbarrier wait is bounded.
+// TMA, warp 1 MMA issue, warps 2..5 the online softmax of one row each (position <= the
+// row's own position and the window only in tiles at those edges, the stream of an
+// intra-stream layer as a bit per column) and the unnormalised partial (O, running max in
+// log2 units, sum) that combine_kernel merges.  Every mbarrier wait is bounded.
+// Bound by HBM and, at small batches, by a CTA's start and end.  Measured, 4 sequences of up
+// to 8192 tokens, 80B heads, intra-stream: this kernel 61 -> 37 us, the step with its append
+// and combine 74 -> 44 us.  Before, per-element masks (three compares and a modular step
+// each) took 4400 of a tile's 7000 cycles; its 128 KB take 5800 at the HBM rate with every
+// SM streaming.
 namespace dectc {
 constexpr int DH = 256, BM = 128, BN = 128, NSLOT = 5, NTHREADS = 192;
 constexpr uint32_t COL_O = 256;
@@ -463,23 +531,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) decode_tc_kernel(const __grid_con
   const size_t pidx = ((size_t)b * a.Hkv + g) * a.nsplit + c;
   float* po = a.part_o + pidx * a.rg * DH;
   float2* pml = a.part_ml + pidx * a.rg;
-  dec::grid_dep_wait();
-  dec::grid_dep_launch();
-  const int T = a.lens[b];
-  int k0 = 0, k1 = 0;
-  if (T >= 1 && T <= a.maxT) {
-    int lo, hi;
-    dec::seq_range(a, T, lo, hi);
-    k0 = lo + c * a.chunk;
-    k1 = min(k0 + a.chunk, hi);
-  }
-  if (k0 >= k1) {  // nothing of this sequence in this split: an empty partial
-    for (int i = threadIdx.x; i < a.M; i += NTHREADS) pml[i] = make_float2(-INFINITY, 0.f);
-    return;
-  }
-  const int nt = (k1 - k0 + BN - 1) / BN, nunits = 4 * nt;
-
-  // rows M..127 of the query tile are zero (their scores are masked; no NaN enters O)
+  // Set-up first: it needs nothing from the kernels before this one.  Rows M..127 of the
+  // query tile are zero (their scores are finite and their results are not stored).
   for (int i = threadIdx.x; i < (DH / 64) * (BM - a.M) * 8; i += NTHREADS) {
     const int blk = i / ((BM - a.M) * 8), rem = i % ((BM - a.M) * 8);
     reinterpret_cast<uint4*>(sm.q[blk] + (a.M + rem / 8) * 64)[rem % 8] = make_uint4(0, 0, 0, 0);
@@ -504,10 +557,21 @@ __global__ void __launch_bounds__(NTHREADS, 1) decode_tc_kernel(const __grid_con
     tmem_alloc(&sm.tmem_base, 512);
     tmem_relinquish();
   }
+  dec::grid_dep_wait();
+  dec::grid_dep_launch();
+  const int T = a.lens[b];
+  int k0, k1;
+  dec::split_range(a, T, c, BN, k0, k1);
+  const int nt = (k1 - k0 + BN - 1) / BN, nunits = 4 * nt;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
+  if (k0 >= k1) {  // nothing of this sequence in this split: an empty partial
+    for (int i = threadIdx.x; i < a.M; i += NTHREADS) pml[i] = make_float2(-INFINITY, 0.f);
+    if (warp == 0) tmem_dealloc(tmem, 512);
+    return;
+  }
   volatile int* abort = &sm.abort;
 
   if (warp == 0) {
@@ -614,6 +678,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) decode_tc_kernel(const __grid_con
     const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16);
     const uint32_t tO = tl + COL_O;
     const float c2 = a.scale_log2;
+    const int own_lo = (T - 1) * a.n;                                             // first position of the new token
+    const int win_hi = a.mode == SFA_LOCAL ? T * a.n - 1 - a.window : -1;  // outside some row's window up to here
+    // n divides 32: columns of the row's stream repeat from word to word and tile to tile
+    // (a split starts at a multiple of BN)
+    uint32_t stream_word = 0;
+    if (a.mode == SFA_WITHIN && 32 % a.n == 0)
+      for (int e = (s + a.n - k0 % a.n) % a.n; e < 32; e += a.n) stream_word |= 1u << e;
     float m_run = -INFINITY, l_run = 0.f;
     bool ok = true;
     for (int i = 0; i < nt; ++i) {
@@ -627,19 +698,30 @@ __global__ void __launch_bounds__(NTHREADS, 1) decode_tc_kernel(const __grid_con
 #pragma unroll
       for (int cc = 0; cc < BN / 32; ++cc) tmem_ld32(tS + cc * 32, reinterpret_cast<uint32_t*>(x) + cc * 32);
       tmem_ld_wait();
-      {
-        const int base = k0 + i * BN;
-        // (position - s) mod n, stepped along the columns (intra-stream layers keep 0)
-        int kres = (base - s) % a.n;
-        if (kres < 0) kres += a.n;
-        const int lim = min(k1 - 1, pq), wlo = a.mode == SFA_LOCAL ? pq - a.window : -1;
-        const bool within = a.mode == SFA_WITHIN;
+      const int base = k0 + i * BN;
+      // the tile that reaches the new token's own positions or the split's end, and (LOCAL)
+      // those at the rows' window edges
+      if (base + BN - 1 > own_lo || base + BN > k1 || base <= win_hi) {
+        const int e_hi = min(k1 - 1, pq) - base, e_lo = a.mode == SFA_LOCAL ? pq - a.window + 1 - base : 0;
 #pragma unroll
-        for (int e = 0; e < BN; ++e) {
-          const int p = base + e;
-          if (!rv || p > lim || p <= wlo || (within && kres != 0)) x[e] = -INFINITY;
-          kres = kres + 1 == a.n ? 0 : kres + 1;
+        for (int e = 0; e < BN; ++e)
+          if (e > e_hi || e < e_lo) x[e] = -INFINITY;
+      }
+      if (a.mode == SFA_WITHIN && a.n > 1) {
+        // the stream condition as one bit per column
+        uint32_t vis[4] = {stream_word, stream_word, stream_word, stream_word};
+        if (stream_word == 0) {  // n does not divide 32: the pattern shifts from tile to tile
+          int e = (base - s) % a.n;  // first column of the row's stream
+          e = e <= 0 ? -e : a.n - e;
+          for (; e < BN; e += a.n) {
+#pragma unroll
+            for (int w = 0; w < 4; ++w)
+              if ((e >> 5) == w) vis[w] |= 1u << (e & 31);
+          }
         }
+#pragma unroll
+        for (int e = 0; e < BN; ++e)
+          if (!((vis[e >> 5] >> (e & 31)) & 1u)) x[e] = -INFINITY;
       }
       float mx[8];
 #pragma unroll
@@ -701,18 +783,26 @@ __global__ void __launch_bounds__(NTHREADS, 1) decode_tc_kernel(const __grid_con
     }
     if (ok && __all_sync(0xffffffffu, mbar_wait(&sm.pv_done, (nt - 1) & 1, abort, a.status))) {
       tc_fence_after();
-      float* orow = po + (size_t)row * DH;
-#pragma unroll 1
+      // the partial rows leave through shared memory (the ring is no longer read), 32 columns
+      // at a time: 16-byte units XOR-swizzled by the row, then 128 bytes of four rows per store
+      uint8_t* stg = reinterpret_cast<uint8_t*>(sm.ring[0][0]) + q4 * 8192;
+#pragma unroll 2
       for (int cc = 0; cc < DH / 32; ++cc) {
         uint32_t o[32];
         tmem_ld32(tO + cc * 32, o);
         tmem_ld_wait();
-        if (rv) {
+        uint8_t* buf = stg + (cc & 1) * 4096;
 #pragma unroll
-          for (int e = 0; e < 32; e += 4)
-            *reinterpret_cast<float4*>(orow + cc * 32 + e) =
-                make_float4(__uint_as_float(o[e]), __uint_as_float(o[e + 1]), __uint_as_float(o[e + 2]),
-                            __uint_as_float(o[e + 3]));
+        for (int u = 0; u < 8; ++u)
+          *reinterpret_cast<uint4*>(buf + lane * 128 + ((u ^ (lane & 7)) << 4)) =
+              make_uint4(o[4 * u], o[4 * u + 1], o[4 * u + 2], o[4 * u + 3]);
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int rr = k * 4 + (lane >> 3), u = lane & 7;
+          if (q4 * 32 + rr < a.M)
+            *reinterpret_cast<uint4*>(po + (size_t)(q4 * 32 + rr) * DH + cc * 32 + u * 4) =
+                *reinterpret_cast<const uint4*>(buf + rr * 128 + ((u ^ (rr & 7)) << 4));
         }
       }
       if (rv) pml[row] = make_float2(m_run * c2, l_run);
@@ -759,7 +849,6 @@ DecodePlan decode_plan(int B, int maxT, int n, int Hq, int Hkv, int Dh, int mode
     }
   }
   const long long tiles_per = (tiles + best - 1) / best;
-  p.chunk = (int)(tiles_per * KT);
   p.nsplit = (int)((tiles + tiles_per - 1) / tiles_per);
   const size_t parts = (size_t)B * Hkv * p.ngroups * p.nsplit;
   p.part_o_bytes = parts * p.rg * Dh * sizeof(float);
@@ -787,7 +876,7 @@ static cudaError_t launch_decode_t(const dec::DecodeArgs& a, cudaStream_t st) {
   cfg.numAttrs = 1;
   e = cudaLaunchKernelEx(&cfg, decode_kernel<DH, MT>, a);
   if (e != cudaSuccess) return e;
-  cfg.gridDim = dim3(a.Hkv * a.ngroups, a.B, (DH / 8) * ((std::min(a.rg, a.M) + 7) / 8));
+  cfg.gridDim = dim3(std::min(a.rg, a.M), a.Hkv * a.ngroups, a.B);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = 0;
   return cudaLaunchKernelEx(&cfg, combine_kernel<DH>, a);
@@ -824,7 +913,7 @@ static cudaError_t launch_decode_tc(const dec::DecodeArgs& a, cudaStream_t st) {
   cfg.numAttrs = 1;
   e = cudaLaunchKernelEx(&cfg, decode_tc_kernel, p);
   if (e != cudaSuccess) return e;
-  cfg.gridDim = dim3(a.Hkv, a.B, (DH / 8) * ((std::min(a.rg, a.M) + 7) / 8));
+  cfg.gridDim = dim3(a.M, a.Hkv, a.B);
   cfg.blockDim = dim3(256);
   cfg.dynamicSmemBytes = 0;
   return cudaLaunchKernelEx(&cfg, dec::combine_kernel<DH>, a);
@@ -854,11 +943,11 @@ cudaError_t launch_sfa_decode(const void* q, const void* kc, const void* vc, con
   a.M = p.M;
   a.ngroups = p.ngroups;
   a.nsplit = p.nsplit;
-  a.chunk = p.chunk;
   a.rg = p.rg;
   a.mode = mode;
   a.window = window;
   a.scale_log2 = scale * 1.4426950408889634f;
+  a.d_nsplit = make_fast_div((uint32_t)p.nsplit);
   if (p.tc) return launch_decode_tc(a, st);
   const bool two = p.M > 16;  // a row group of more than 16 rows takes two m16 tiles
   if (Dh == 64) return two ? launch_decode_t<64, 2>(a, st) : launch_decode_t<64, 1>(a, st);
@@ -869,9 +958,17 @@ cudaError_t launch_sfa_decode(const void* q, const void* kc, const void* vc, con
 cudaError_t launch_kv_append(const void* kn, const void* vn, void* kc, void* vc, const int32_t* lens, int B,
                              int Lcap, int n, int Hkv, int Dh, int32_t* status, cudaStream_t st) {
   const long long warps = (long long)B * n;
-  dec::append_kernel<<<(unsigned)((warps * 32 + 255) / 256), 256, 0, st>>>(
-      (const uint4*)kn, (const uint4*)vn, (uint4*)kc, (uint4*)vc, lens, B, Lcap, n, Hkv * Dh / 8, status);
-  return cudaGetLastError();
+  cudaLaunchAttribute pdl[1];
+  pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  pdl[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((warps * 32 + 255) / 256));
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cfg.attrs = pdl;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, dec::append_kernel, (const uint4*)kn, (const uint4*)vn, (uint4*)kc, (uint4*)vc, lens, B,
+                            Lcap, n, Hkv * Dh / 8, status);
 }
 
 }  // namespace hdsfa
