@@ -5,7 +5,8 @@
 //           position p = r*ns + s and Lvp = row_terms_pitch(Lv), so one query tile
 //           of any stream is contiguous floats (a single bulk copy).  Negated so the
 //           backward folds them in with one add / fused multiply-add.  Rows in
-//           [Lv, Lvp) get -lse2 = -inf and -delta = 0 (their P and dS vanish).
+//           [Lv, Lvp) get -lse2 = -inf and -delta = 0 (their P and dS vanish), from the
+//           same launch (a kernel of their own cost short layers 2 us).
 //           Also zeroes the fp32 dQ accumulator where asked to (sfa_bwd_prep; clear
 //           alone may run on another stream).
 // finalize: dq = bf16(scale * accumulator), round to nearest even.
@@ -39,7 +40,7 @@ __global__ void __launch_bounds__(256) sfa_bwd_prep_kernel(const bf16* __restric
   // warp -> (b, s, r-block, h), h fastest; 32-bit index math (the host caps B*nL*Hq
   // below 2^30)
   const unsigned Hq = (unsigned)g.Hq, ns = (unsigned)g.ns, Lv = (unsigned)g.Lv, nL = (unsigned)g.nL;
-  const unsigned nrb = (Lv + RPW - 1) / RPW;
+  const unsigned nrb = (unsigned)row_terms_pitch(g.Lv) / RPW;  // the padding rows too
   const unsigned w = (unsigned)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if ((long long)w >= (long long)g.B * ns * nrb * Hq) return;
   const unsigned h = w % Hq, w1 = w / Hq, rb = w1 % nrb, w2 = w1 / nrb, s = w2 % ns, b = w2 / ns;
@@ -79,10 +80,10 @@ __global__ void __launch_bounds__(256) sfa_bwd_prep_kernel(const bf16* __restric
       const float v = __shfl_sync(0xffffffffu, acc[i], sb * LPR);
       if (lane == i * RPG + sb) dl = v;
     }
-  if (mine) {
+  if (lane < RPW) {
     const long long t = (bh * ns + s) * row_terms_pitch(g.Lv) + r0 + lane;
-    delta_t[t] = -dl;
-    lse2_t[t] = -lv * 1.4426950408889634f;
+    delta_t[t] = mine ? -dl : 0.f;
+    lse2_t[t] = mine ? -lv * 1.4426950408889634f : -INFINITY;
   }
   if (ZERO) {  // this warp's rows of the dQ accumulator, DH contiguous floats each
 #pragma unroll
@@ -100,15 +101,6 @@ __global__ void __launch_bounds__(256) sfa_bwd_prep_kernel(const bf16* __restric
 __global__ void __launch_bounds__(256) sfa_bwd_clear_kernel(float4* __restrict__ acc, long long n4) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x)
     acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-}
-
-__global__ void sfa_bwd_pad_kernel(float* __restrict__ lse2_t, float* __restrict__ delta_t, SfaGeom g) {
-  const int Lvp = row_terms_pitch(g.Lv), pad = Lvp - g.Lv;
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)g.B * g.Hq * g.ns * pad) return;
-  const long long t = (i / pad) * Lvp + g.Lv + i % pad;
-  lse2_t[t] = -INFINITY;
-  delta_t[t] = 0.f;
 }
 
 __global__ void __launch_bounds__(256) sfa_bwd_finalize_kernel(const float* __restrict__ dq_acc,
@@ -129,7 +121,7 @@ __global__ void __launch_bounds__(256) sfa_bwd_finalize_kernel(const float* __re
 cudaError_t launch_sfa_bwd_prep(const void* o, const void* dout, const float* lse, float* lse2_ws,
                                 float* delta_ws, float* dq_ws, const SfaGeom& g, int Dh,
                                 cudaStream_t st, bool zero) {
-  const long long warps = (long long)g.B * g.ns * ((g.Lv + 7) / 8) * g.Hq;  // 8 rows of one problem each
+  const long long warps = (long long)g.B * g.ns * (row_terms_pitch(g.Lv) / 8) * g.Hq;  // 8 rows of one problem each
   const unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
   const bf16 *ob = (const bf16*)o, *db = (const bf16*)dout;
   if (Dh == 256) {
@@ -148,15 +140,7 @@ cudaError_t launch_sfa_bwd_prep(const void* o, const void* dout, const float* ls
     else
       sfa_bwd_prep_kernel<128, false><<<blocks, 256, 0, st>>>(ob, db, lse, lse2_ws, delta_ws, dq_ws, g);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const int pad = row_terms_pitch(g.Lv) - g.Lv;
-  if (pad > 0) {
-    const long long n = (long long)g.B * g.Hq * g.ns * pad;
-    sfa_bwd_pad_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(lse2_ws, delta_ws, g);
-    e = cudaGetLastError();
-  }
-  return e;
+  return cudaGetLastError();
 }
 
 cudaError_t launch_sfa_bwd_clear(float* dq_ws, const SfaGeom& g, int Dh, cudaStream_t st) {
