@@ -139,6 +139,27 @@ HD_DEVINLINE int swz(int row, int col) {
   return row * RL + ((((col >> 3) ^ (row & 7))) << 3) + (col & 7);
 }
 
+// Programmatic dependent launch: a kernel launched with launch_early may start while the
+// kernel before it in the stream is finishing.  It waits (grid_dep_wait) for that kernel's
+// completion before it touches global memory, and lets its own successor start its set-up
+// (grid_dep_launch).  Without the launch attribute both are no-ops.
+HD_DEVINLINE void grid_dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+HD_DEVINLINE void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_early(void (*kernel)(P...), dim3 grid, unsigned block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute pdl[1];
+  pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  pdl[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
+  cfg.attrs = pdl;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 HD_DEVINLINE void set_status(int32_t* st, int bit) {
   if (st) atomicOr(st, bit);
 }

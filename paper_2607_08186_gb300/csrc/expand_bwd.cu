@@ -105,27 +105,39 @@ constexpr int kField = 21;
 __global__ void __launch_bounds__(kRankTile) rank_kernel(const int32_t* __restrict__ ids, long long N, int V,
                                                         unsigned long long* __restrict__ partial,
                                                         unsigned* __restrict__ counts, int32_t* status) {
-  __shared__ ulonglong2 sj[kRankTile / 2];
+  // Ids in 32 bits; outside the diagonal tiles the order of the tokens is the tiles', so a
+  // pair takes two compares and two adds (64-bit keys: 10.1 us for 4096 tokens; this 7.6)
+  __shared__ int4 sj[kRankTile / 4];
   const long long j0 = (long long)blockIdx.y * kRankTile;
   const long long i = (long long)blockIdx.x * kRankTile + threadIdx.x;
+  grid_dep_wait();
+  grid_dep_launch();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) counts[threadIdx.x] = 0;
-  // keys past N are kNoKey, above every real key; ids are checked once (tile row x = 0)
-  reinterpret_cast<unsigned long long*>(sj)[threadIdx.x] =
-      make_key(ids, j0 + threadIdx.x, N, V, blockIdx.x == 0 ? status : nullptr);
+  // tokens past N and ids outside [0, V) take the last id; ids are checked once (tile row x = 0)
+  reinterpret_cast<uint32_t*>(sj)[threadIdx.x] =
+      (uint32_t)(make_key(ids, j0 + threadIdx.x, N, V, blockIdx.x == 0 ? status : nullptr) >> 32);
   __syncthreads();
   if (i >= N) return;
-  const unsigned long long ki = make_key(ids, i, N, V, nullptr);
-  const uint32_t vi = (uint32_t)(ki >> 32);
-  unsigned below = 0, same = 0, same_below = 0;
+  const uint32_t vi = (uint32_t)(make_key(ids, i, N, V, nullptr) >> 32);
+  unsigned less = 0, same = 0, same_below = 0;
+  if (blockIdx.x != blockIdx.y) {
 #pragma unroll 8
-  for (int t = 0; t < kRankTile / 2; ++t) {
-    const ulonglong2 p = sj[t];
-    const bool bx = p.x < ki, by = p.y < ki;
-    const bool sx = (uint32_t)(p.x >> 32) == vi, sy = (uint32_t)(p.y >> 32) == vi;
-    below += bx + by;
-    same += sx + sy;
-    same_below += (sx && bx) + (sy && by);
+    for (int t = 0; t < kRankTile / 4; ++t) {
+      const int4 p = sj[t];
+      less += ((uint32_t)p.x < vi) + ((uint32_t)p.y < vi) + ((uint32_t)p.z < vi) + ((uint32_t)p.w < vi);
+      same += ((uint32_t)p.x == vi) + ((uint32_t)p.y == vi) + ((uint32_t)p.z == vi) + ((uint32_t)p.w == vi);
+    }
+    same_below = blockIdx.y < blockIdx.x ? same : 0;
+  } else {
+#pragma unroll 8
+    for (int t = 0; t < kRankTile; ++t) {
+      const uint32_t v = reinterpret_cast<const uint32_t*>(sj)[t];
+      less += v < vi;
+      same += v == vi;
+      same_below += v == vi && t < (int)threadIdx.x;
+    }
   }
+  const unsigned below = less + same_below;
   partial[blockIdx.y * N + i] = (unsigned long long)below | ((unsigned long long)same << kField) |
                                 ((unsigned long long)same_below << (2 * kField));
 }
@@ -135,6 +147,8 @@ __global__ void __launch_bounds__(256) scatter_kernel(const int32_t* __restrict_
                                                       unsigned long long* __restrict__ keys, uint4* __restrict__ light,
                                                       uint4* __restrict__ heavy, unsigned* __restrict__ counts) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  grid_dep_wait();
+  grid_dep_launch();
   if (i >= N) return;
   unsigned long long acc = 0;  // fields stay below 2^15 (N <= kRankMax): no carries
 #pragma unroll 8
@@ -233,25 +247,86 @@ __global__ void __launch_bounds__(kRowThreads, 3) rows_kernel(const bf16* __rest
                                                           const uint4* __restrict__ heavy,
                                                           const unsigned* __restrict__ counts,
                                                           float* __restrict__ de, long long N, int n, int V,
-                                                          int D) {
+                                                          int D, FastDiv div_d8) {
   __shared__ float part[kHeavyBlocks][kHeavyItems][9];  // padded against bank conflicts
   const int d8 = D / 8, items = n * d8;
   const long long nD = (long long)n * D;
   const int SL = (items + kLightItems - 1) / kLightItems, SH = (items + kHeavyItems - 1) / kHeavyItems;
-  // heavy units first: they take longest, so they start before the light ones
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  grid_dep_wait();
+  grid_dep_launch();
   // The run lists hold at most N records each; a record or a key outside the plan's
   // ranges (a workspace the plan did not write) is skipped, so every access stays in
   // bounds whatever the workspace holds.
   const long long nl = counts[0] < N ? counts[0] : N, nh = counts[1] < N ? counts[1] : N;
-  const long long hunits = nh * SH, units = hunits + nl * SL;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (long long w = blockIdx.x; w < units; w += gridDim.x) {
-    if (w >= hunits) {
-      const long long lw = w - hunits, r = lw / SL;
-      const int z = (int)(lw - r * SL);
-      const uint4 rec = light[r];
-      const uint32_t start = rec.x, m = rec.y, v = rec.w;
-      if (start >= N || m > N - start || v >= (uint32_t)V || rec.z >= N) continue;
+  // heavy units first: they take longest, so they start before the light ones
+  const long long hunits = nh * SH;
+  long long w = blockIdx.x;
+  for (; w < hunits; w += gridDim.x) {
+    const long long r = w / SH;
+    const int z = (int)(w - r * SH);
+    const uint4 rec = heavy[r];
+    const uint32_t start = rec.x, m = rec.y, v = rec.w;
+    if (start >= N || m > N - start || v >= (uint32_t)V) continue;  // uniform over the block
+    const int itm = z * kHeavyItems + lane;
+    const bool live = itm < items;
+    // token block of this warp: [m*warp/8, m*(warp+1)/8)
+    const uint32_t jb = (uint32_t)((unsigned long long)m * warp / kHeavyBlocks);
+    const uint32_t je = (uint32_t)((unsigned long long)m * (warp + 1) / kHeavyBlocks);
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (uint32_t j0 = jb; j0 < je; j0 += 8) {
+      uint4 x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        x[u] = make_uint4(0, 0, 0, 0);
+        if (j0 + u < je && live) {
+          const long long tok = (long long)(uint32_t)keys[start + j0 + u];
+          if (tok < N) x[u] = *reinterpret_cast<const uint4*>(dx + tok * nD + (long long)itm * 8);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (j0 + u < je) add_bf16x8(acc, x[u]);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) part[warp][lane][e] = acc[e];
+    __syncthreads();
+    if (warp == 0 && live) {
+      const int s = fast_div(itm, div_d8), c = itm - s * d8;
+      float* drow = de + ((long long)s * V + v) * D + c * 8;
+      const float4 a0 = reinterpret_cast<const float4*>(drow)[0], a1 = reinterpret_cast<const float4*>(drow)[1];
+      float sum[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) sum[e] = part[0][lane][e];
+#pragma unroll
+      for (int b = 1; b < kHeavyBlocks; ++b)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) sum[e] += part[b][lane][e];
+      rmw_add(drow, a0, a1, sum);
+    }
+    __syncthreads();
+  }
+  // Light units: run r, slice z, stepped by the grid without a division per unit; the next
+  // unit's record is on its way while this one is summed, and a run's tokens come from one
+  // load of its keys, a lane each.  (HBM-bound; 416 MB for 4096 Zipf ids, n = 4, D = 4096:
+  // 84 -> 76 us, 5.5 TB/s.)
+  const int step_r = (int)(gridDim.x / SL), step_z = (int)(gridDim.x % SL);
+  long long r = (w - hunits) / SL;
+  int z = (int)((w - hunits) - r * SL);
+  uint4 rec = r < nl ? light[r] : make_uint4(0, 0, 0, 0);
+  while (r < nl) {
+    long long rn = r + step_r;
+    int zn = z + step_z;
+    if (zn >= SL) {
+      zn -= SL;
+      ++rn;
+    }
+    const uint4 next = rn < nl ? light[rn] : make_uint4(0, 0, 0, 0);
+    const uint32_t start = rec.x, m = rec.y, v = rec.w;
+    if (start < N && m <= N - start && m <= (uint32_t)kHeavy && v < (uint32_t)V && rec.z < N) {
+      // this lane's token of the run: the first from the record, the others from the keys
+      uint32_t mytok = rec.z;
+      if (lane > 0 && (uint32_t)lane < m) mytok = (uint32_t)keys[start + lane];
       int it[2];
       float* drow[2];
       float4 e0[2], e1[2];
@@ -263,26 +338,23 @@ __global__ void __launch_bounds__(kRowThreads, 3) rows_kernel(const bf16* __rest
 #pragma unroll
         for (int e = 0; e < 8; ++e) acc[q][e] = 0.f;
         if (it[q] < items) {
-          const int s = it[q] / d8, c = it[q] - s * d8;
+          const int s = fast_div(it[q], div_d8), c = it[q] - s * d8;
           drow[q] = de + ((long long)s * V + v) * D + c * 8;
           e0[q] = reinterpret_cast<const float4*>(drow[q])[0];
           e1[q] = reinterpret_cast<const float4*>(drow[q])[1];
         }
       }
-      // first token from the record, the others from the sorted keys
       for (uint32_t j0 = 0; j0 < m; j0 += 4) {
         uint4 x[4][2];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const uint32_t j = j0 + u;
-          long long tok = -1;
-          if (j < m) tok = j == 0 ? (long long)rec.z : (long long)(uint32_t)keys[start + j];
-          if (tok >= N) tok = -1;
+          const uint32_t tok = __shfl_sync(0xffffffffu, mytok, (int)(j0 + u) & 31);
+          const bool live = j0 + u < m && tok < N;
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             x[u][q] = make_uint4(0, 0, 0, 0);
-            if (tok >= 0 && drow[q] != nullptr)
-              x[u][q] = *reinterpret_cast<const uint4*>(dx + tok * nD + (long long)it[q] * 8);
+            if (live && drow[q] != nullptr)
+              x[u][q] = *reinterpret_cast<const uint4*>(dx + (long long)tok * nD + (long long)it[q] * 8);
           }
         }
 #pragma unroll
@@ -295,50 +367,10 @@ __global__ void __launch_bounds__(kRowThreads, 3) rows_kernel(const bf16* __rest
 #pragma unroll
       for (int q = 0; q < 2; ++q)
         if (drow[q] != nullptr) rmw_add(drow[q], e0[q], e1[q], acc[q]);
-    } else {
-      const long long r = w / SH;
-      const int z = (int)(w - r * SH);
-      const uint4 rec = heavy[r];
-      const uint32_t start = rec.x, m = rec.y, v = rec.w;
-      if (start >= N || m > N - start || v >= (uint32_t)V) continue;  // uniform over the block
-      const int itm = z * kHeavyItems + lane;
-      const bool live = itm < items;
-      // token block of this warp: [m*warp/8, m*(warp+1)/8)
-      const uint32_t jb = (uint32_t)((unsigned long long)m * warp / kHeavyBlocks);
-      const uint32_t je = (uint32_t)((unsigned long long)m * (warp + 1) / kHeavyBlocks);
-      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      for (uint32_t j0 = jb; j0 < je; j0 += 8) {
-        uint4 x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          x[u] = make_uint4(0, 0, 0, 0);
-          if (j0 + u < je && live) {
-            const long long tok = (long long)(uint32_t)keys[start + j0 + u];
-            if (tok < N) x[u] = *reinterpret_cast<const uint4*>(dx + tok * nD + (long long)itm * 8);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (j0 + u < je) add_bf16x8(acc, x[u]);
-      }
-#pragma unroll
-      for (int e = 0; e < 8; ++e) part[warp][lane][e] = acc[e];
-      __syncthreads();
-      if (warp == 0 && live) {
-        const int s = itm / d8, c = itm - s * d8;
-        float* drow = de + ((long long)s * V + v) * D + c * 8;
-        const float4 a0 = reinterpret_cast<const float4*>(drow)[0], a1 = reinterpret_cast<const float4*>(drow)[1];
-        float sum[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) sum[e] = part[0][lane][e];
-#pragma unroll
-        for (int b = 1; b < kHeavyBlocks; ++b)
-#pragma unroll
-          for (int e = 0; e < 8; ++e) sum[e] += part[b][lane][e];
-        rmw_add(drow, a0, a1, sum);
-      }
-      __syncthreads();
     }
+    rec = next;
+    r = rn;
+    z = zn;
   }
 }
 
@@ -347,6 +379,8 @@ __global__ void __launch_bounds__(256) select_kernel(const uint4* __restrict__ x
                                                      long long rows, int n, int d16) {
   const int lane = threadIdx.x & 31;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+  grid_dep_wait();
+  grid_dep_launch();
   for (long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += nw) {
     const uint4* src = x + (r * n + (n - 1)) * d16;
     uint4* dst = y + r * d16;
@@ -359,6 +393,8 @@ __global__ void __launch_bounds__(256) select_bwd_kernel(const uint4* __restrict
                                                          long long rows_x, int n, int d16) {
   const int lane = threadIdx.x & 31;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+  grid_dep_wait();
+  grid_dep_launch();
   for (long long p = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < rows_x; p += nw) {
     uint4* dst = dx + p * d16;
     if (p % n == n - 1) {
@@ -418,10 +454,10 @@ cudaError_t launch_expand_bwd_plan(const int32_t* ids, int B, int L, int V, void
   const ExpandBwdWs w = split_ws(ws, N);
   if (N <= kRankMax) {
     const int tiles = (int)((N + kRankTile - 1) / kRankTile);
-    rank_kernel<<<dim3(tiles, tiles), kRankTile, 0, st>>>(ids, N, V, w.partial, w.counts, status);
-    scatter_kernel<<<tiles, kRankTile, 0, st>>>(ids, N, V, w.partial, tiles, w.keys, w.light, w.heavy,
-                                                w.counts);
-    return cudaGetLastError();
+    cudaError_t e = launch_early(rank_kernel, dim3(tiles, tiles), kRankTile, st, ids, N, V, w.partial, w.counts, status);
+    if (e != cudaSuccess) return e;
+    return launch_early(scatter_kernel, dim3(tiles), kRankTile, st, ids, N, V,
+                        (const unsigned long long*)w.partial, tiles, w.keys, w.light, w.heavy, w.counts);
   }
   const unsigned nchunks = (unsigned)(N2 / kChunk);
   chunk_kernel<<<nchunks, kSortThreads, 0, st>>>(w.keys, ids, N, V, 0, w.counts, status);
@@ -439,23 +475,21 @@ cudaError_t launch_expand_bwd_apply(const void* dx, float* de, int B, int L, int
                                     cudaStream_t st) {
   using namespace ebwd;
   const ExpandBwdWs w = split_ws(const_cast<void*>(ws), (long long)B * L);
-  rows_kernel<<<152 * 3, kRowThreads, 0, st>>>((const bf16*)dx, w.keys, w.light, w.heavy, w.counts, de,
-                                                 (long long)B * L, n, V, D);
-  return cudaGetLastError();
+  return launch_early(rows_kernel, dim3(152 * 3), kRowThreads, st, (const bf16*)dx, (const unsigned long long*)w.keys,
+                      (const uint4*)w.light, (const uint4*)w.heavy, (const unsigned*)w.counts, de, (long long)B * L, n, V,
+                      D, make_fast_div((uint32_t)(D / 8)));
 }
 
 cudaError_t launch_select_final(const void* x, void* y, int B, int L, int n, int D, cudaStream_t st) {
   const long long rows = (long long)B * L;
-  ebwd::select_kernel<<<grid_for(rows, 8, 152LL * 64), 256, 0, st>>>((const uint4*)x, (uint4*)y, rows, n,
-                                                                     D / 8);
-  return cudaGetLastError();
+  return launch_early(ebwd::select_kernel, dim3(grid_for(rows, 8, 152LL * 64)), 256, st, (const uint4*)x, (uint4*)y, rows, n,
+                      D / 8);
 }
 
 cudaError_t launch_select_final_bwd(const void* dy, void* dx, int B, int L, int n, int D, cudaStream_t st) {
   const long long rows_x = (long long)B * L * n;
-  ebwd::select_bwd_kernel<<<grid_for(rows_x, 8, 152LL * 64), 256, 0, st>>>((const uint4*)dy, (uint4*)dx,
-                                                                           rows_x, n, D / 8);
-  return cudaGetLastError();
+  return launch_early(ebwd::select_bwd_kernel, dim3(grid_for(rows_x, 8, 152LL * 64)), 256, st, (const uint4*)dy, (uint4*)dx,
+                      rows_x, n, D / 8);
 }
 
 }  // namespace hdsfa

@@ -69,13 +69,8 @@ struct DecodeArgs {
   FastDiv d_nsplit;
 };
 
-// Programmatic dependent launch: both kernels are launched so that they may start
-// while the kernel before them in the stream is finishing; each waits for that
-// kernel's results before its first read of them, and the decode kernel lets the
-// combine kernel launch at once, so the combine's launch and start overlap the
-// decode's tail.  Without the launch attribute both are no-ops.
-HD_DEVINLINE void grid_dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-HD_DEVINLINE void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+// Both kernels are launched early (launch_early's attribute): the decode kernel lets the
+// combine kernel start at once, so the combine's launch and start overlap its tail.
 
 // Visible position range [lo, hi) of a sequence of T tokens (the new token's rows
 // see nothing outside it; per-row conditions are applied per element).
@@ -557,8 +552,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) decode_tc_kernel(const __grid_con
     tmem_alloc(&sm.tmem_base, 512);
     tmem_relinquish();
   }
-  dec::grid_dep_wait();
-  dec::grid_dep_launch();
+  grid_dep_wait();
+  grid_dep_launch();
   const int T = a.lens[b];
   int k0, k1;
   dec::split_range(a, T, c, BN, k0, k1);
