@@ -102,49 +102,6 @@ struct Params {
   int32_t* status;
 };
 
-// Arrive on the barrier at the same place in the pair's first CTA.
-HD_DEVINLINE uint32_t lead_addr(const void* p) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, 0;\n" : "=r"(r) : "r"(smem_u32(p)));
-  return r;
-}
-HD_DEVINLINE void arrive_lead(uint32_t lead_bar) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];\n" ::"r"(lead_bar) : "memory");
-}
-// Load into this CTA's shared memory, counted on the first CTA's barrier.
-HD_DEVINLINE void tma_load_pair(void* dst, const CUtensorMap* m, uint32_t lead_bar, int c0, int c1, int c2, int c3,
-                                int c4) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5, %6, %7}], [%2];\n" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(m)), "r"(lead_bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
-      : "memory");
-}
-HD_DEVINLINE void mma2_ss(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
-  asm volatile(
-      "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
-      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accum));
-}
-HD_DEVINLINE void mma2_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
-  asm volatile(
-      "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
-      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
-      "r"(a), "l"(b), "r"(idesc), "r"(accum));
-}
-// Arrive on `bar` of both CTAs once every MMA issued so far has completed.
-HD_DEVINLINE void commit2(uint64_t* bar) {
-  asm volatile(
-      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
-      " @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}\n" ::
-          "r"(smem_u32(bar)),
-      "h"((uint16_t)3)
-      : "memory");
-}
-HD_DEVINLINE void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;\n" ::: "memory");
-}
-
 // One work item: its kind, stationary rows and the streamed steps.
 struct Item {
   int kind;
@@ -262,10 +219,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
     fence_mbar_init();
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&sm.tmem_base)),
-                 "r"(512)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
+    tmem_alloc_pair(&sm.tmem_base, 512);
   }
   tc_fence_before();
   __syncthreads();
@@ -689,7 +643,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
   cluster_sync();  // neither CTA's barriers or TMEM are used any more
   if (warp == 0) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512) : "memory");
+    tmem_dealloc_pair(tmem, 512);
   }
 }
 // Head chunks: dv / dk rows (bf16) from the chunks' fp32 partial sums, added in chunk
