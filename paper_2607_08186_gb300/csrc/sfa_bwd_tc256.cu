@@ -23,18 +23,20 @@
 // with the fused form before (one CTA per key tile and head-dim half, S and dP computed
 // by both halves, dQ added into an fp32 accumulator by TMA reduce: 3.34 ms of it, about
 // 4900 cycles per 128 x 64 tile against 3250 of its shared-memory traffic), 2.85 ms with
-// this one (2.1 ms); final-stream CROSS layer of the same heads 3.84 -> 2.49 ms.  A step
-// takes about 2500 (DV) and 3500 to 4200 (DQ, DK) cycles: what is left over the MMAs is
-// the chain dP complete -> dS -> out issued (about 1800 cycles through two cross-CTA
-// signals, 1024 of them under S(t+1)).
+// this one (2.1 ms); final-stream CROSS layer of the same heads 3.84 -> 2.49 ms.
+// A step takes 2110 (DV), 3100 (DQ) and 3590 (DK) cycles.  With the ring in half tiles, so
+// two waits and two commits per operand in the issuer, it was 2480, 3110 and 4110: a wait
+// takes about 100 cycles, 215 right after a commit, and the few MMAs queued ahead do not
+// cover several in a row (2.76 -> 2.66 ms, the forward included).  What is left in DK is the
+// latency of its Q and dO tiles, of which the ring holds one step (3190 with every load of the same
+// tile), and the row terms' loads.  Streaming the query tiles of all heads from the last
+// tile down, so that the CTAs of a group share them in L2, gained nothing (0.97 to 1.0x).
 //
 // A pair's work item (cluster of two CTAs, 320 threads each, one CTA per SM):
 //   A1, A2   stationary operands, 128 rows x 256 per CTA (DV: A1 only), loaded once
-//   ring     streamed operands in 16 KB pieces of 64 rows x 128 columns, in the order
-//            the issuer consumes them.  As B of S and dP (K-major, N = 128) CTA r holds
-//            streamed rows [64r, 64r+64), two pieces over the head dim; as B of the
-//            output GEMM (MN-major, N = 256) it holds head-dim columns [128r, 128r+128),
-//            two pieces over the rows.
+//   ring     streamed operands in 32 KB slots, in the order the issuer consumes them.  As
+//            B of S and dP (K-major, N = 128) CTA r holds streamed rows [64r, 64r+64); as
+//            B of the output GEMM (MN-major, N = 256) head-dim columns [128r, 128r+128).
 //   TMEM     output in columns 256..511; DQ, DK: S in 0..127, dP in 128..255 (dS packed
 //            bf16 over it, each 64-column half at the start of its own columns); DV: S
 //            double-buffered in 0..255 (P^T packed over its buffer likewise).
@@ -42,10 +44,10 @@
 //            softmax takes S(t+1) into registers while out(t) and dP(t+1) run and dP(t+1)
 //            while S(t+2) runs, so the pipe does not wait for it.
 //            DV: S(0), then per step t: S(t+1) out(t).
-// Roles per CTA: warp 0 TMA producer (+ TMEM owner); warp 1 MMA issuer (the pair's first
-// CTA only: the whole warp runs the loop, one elected lane issues); warps 2..9 softmax,
-// two threads per stationary row (TMEM lane), each half of the streamed columns.  A full barrier lives in the first CTA
-// and counts both CTAs' bytes; commits are multicast to both CTAs.
+// Roles per CTA: warp 0 TMA producer; warp 1 MMA issuer (the pair's first CTA only: the
+// whole warp runs the loop, one elected lane issues) and TMEM owner; warps 2..9 softmax, two
+// threads per stationary row (TMEM lane), each half of the streamed columns.  A full barrier
+// lives in the first CTA and counts both CTAs' bytes; commits are multicast to both CTAs.
 // DQ's two 128-row tiles are the same rows of two heads of one K/V group where the group
 // has an even number of heads (same key range), else consecutive tiles of one head; DK's
 // and DV's are consecutive key tiles.
@@ -64,16 +66,17 @@ typedef __nv_bfloat16 bf16;
 
 namespace tcbwd256 {
 constexpr int BM = 128, BN = 128, DH = 256, NTHREADS = 320;
-constexpr int PR = 64, PC = 128;               // a ring piece: rows x columns
+constexpr int PR = 64, PC = 128;               // rows of a TMA box; head-dim columns of a CTA's output B half
 constexpr int HB = 64;                         // streamed columns of one softmax thread
-constexpr int NSLOT = 6, NSLOT_DV = 10;        // DV streams through A2's space as well
+constexpr int SLOT = PR * DH;                  // a ring slot: half of a streamed tile, four [64 rows][64] swizzle blocks
+constexpr int NSLOT = 3, NSLOT_DV = 5;         // DV streams through A2's space as well
 constexpr uint32_t COL_OUT = 256, COL_D = 128;  // output; dP (DV: the second S buffer)
 enum Kind { kDK = 0, kDV = 1, kDQ = 2 };
 
 struct Smem {
   bf16 a1[BM * DH];           // four [128 rows][64] swizzle blocks
-  bf16 a2[BM * DH];           // DV: ring slots 0..3
-  bf16 ring[NSLOT][PR * PC];  // piece: two [64 rows][64] swizzle blocks
+  bf16 a2[BM * DH];           // DV: ring slots 0 and 1
+  bf16 ring[NSLOT][SLOT];
   float nlse2[2][BN];         // DK, DV: -lse*log2(e) of the streamed query tile, by step parity (loaded by bulk copy)
   float ndelta[2][BN];        // DK: -delta of it
   uint64_t full[NSLOT_DV], empty[NSLOT_DV], a1_full, a2_full;
@@ -95,8 +98,11 @@ struct Params {
   bf16* dv;
   float* dkv;   // head chunks > 1: fp32 partial sums [chunks][2][B][q_ns][Lv][Hkv][DH] (dV, dK)
   int hchunks;  // query-head chunks per K/V head
+  int grp, hper;  // query heads per K/V head, and per chunk
   int nkv;      // DK items (= DV items); DQ items follow
   int head_pairs;
+  // DK / DV item -> key-tile pair, chunk, batch, K/V head; DQ item -> rank, batch, head; group
+  FastDiv d_tile, d_hc, d_kns, d_rank, d_hns, d_ns, d_grp;
   SfaGeom g;
   float scale, scale_log2;
   int32_t* status;
@@ -120,13 +126,14 @@ HD_DEVINLINE Item make_item(const Params& P, int idx, int rank) {
   if (it.kind != kDQ) {
     if (it.kind == kDV) idx -= P.nkv;
     const int HC = P.hchunks, per_tile = HC * G.Hkv * G.q_ns * G.B;
-    const int j = idx / per_tile, rem = idx % per_tile;  // key-tile pair slowest
-    it.hc = rem % HC;
-    const int hsb = rem / HC;
-    it.b = hsb / (G.Hkv * G.q_ns);
-    it.kvh = (hsb / G.q_ns) % G.Hkv;
-    it.s = hsb % G.q_ns;
-    const int grp_all = G.Hq / G.Hkv, hper = (grp_all + HC - 1) / HC;
+    const int j = fast_div(idx, P.d_tile), rem = idx - j * per_tile;  // key-tile pair slowest
+    const int hsb = fast_div(rem, P.d_hc);
+    it.hc = rem - hsb * HC;
+    it.b = fast_div(hsb, P.d_kns);
+    const int hs = hsb - it.b * G.Hkv * G.q_ns;
+    it.kvh = fast_div(hs, P.d_ns);
+    it.s = hs - it.kvh * G.q_ns;
+    const int grp_all = P.grp, hper = P.hper;
     it.grp = min(hper, grp_all - it.hc * hper);
     it.h_base = it.kvh * grp_all + it.hc * hper;
     it.head = it.h_base;
@@ -143,12 +150,12 @@ HD_DEVINLINE Item make_item(const Params& P, int idx, int rank) {
     idx -= 2 * P.nkv;
     const int hp = P.head_pairs, rows = hp ? BM : 2 * BM, nh = hp ? G.Hq / 2 : G.Hq;
     const int ntile = (G.Lq + rows - 1) / rows, per_rank = nh * G.q_ns * G.B;
-    const int mt = ntile - 1 - idx / per_rank, hsb = idx % per_rank;
-    it.b = hsb / (nh * G.q_ns);
-    it.s = hsb % G.q_ns;
-    const int hx = (hsb / G.q_ns) % nh;
+    const int tr = fast_div(idx, P.d_rank), mt = ntile - 1 - tr, hsb = idx - tr * per_rank;
+    it.b = fast_div(hsb, P.d_hns);
+    const int hs = hsb - it.b * nh * G.q_ns, hx = fast_div(hs, P.d_ns);
+    it.s = hs - hx * G.q_ns;
     it.head = hp ? 2 * hx + rank : hx;
-    it.kvh = it.head / (G.Hq / G.Hkv);
+    it.kvh = fast_div(it.head, P.d_grp);
     it.h_base = it.head;
     it.grp = 1;
     const int m0 = mt * rows;
@@ -218,14 +225,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
     sm.abort = 0;
     fence_mbar_init();
   }
-  if (warp == 0) {
+  __syncwarp();
+  cluster_arrive();  // the barriers of this CTA are initialised
+  if (warp == 1) {
+    tma_prefetch(&P.tm_q);
+    tma_prefetch(&P.tm_do);
+    tma_prefetch(&P.tm_k);
+    tma_prefetch(&P.tm_v);
     tmem_alloc_pair(&sm.tmem_base, 512);
+    tc_fence_before();
   }
-  tc_fence_before();
-  __syncthreads();
-  cluster_sync();  // both CTAs' barriers are initialised and their TMEM is allocated
-  tc_fence_after();
-  const uint32_t tmem = sm.tmem_base;
+  cluster_wait();
+  uint32_t tmem = 0;
+  if (warp != 0) {  // the producer does not wait for the TMEM allocation
+    named_bar_sync(1, NTHREADS - 32);
+    tc_fence_after();
+    tmem = sm.tmem_base;
+  }
   volatile int* abort = &sm.abort;
   const int nslot = kind == kDV ? NSLOT_DV : NSLOT;
   bf16* const ring0 = kind == kDV ? sm.a2 : sm.ring[0];  // a2 and ring are adjacent
@@ -237,10 +253,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
       const CUtensorMap* tB1 = kind == kDQ ? &P.tm_k : &P.tm_q;
       const CUtensorMap* tB2 = kind == kDQ ? &P.tm_v : &P.tm_do;
       const CUtensorMap* tB3 = kind == kDV ? &P.tm_do : tB1;
-      tma_prefetch(tA1);
-      tma_prefetch(tA2);
-      tma_prefetch(tB1);
-      tma_prefetch(tB2);
       const int ahead = kind == kDQ ? it.head : it.kvh, astr = kind == kDQ ? it.s : it.sk;
       const int bstr = kind == kDQ ? it.sk : it.s;
       auto load_a = [&](bf16* dst, const CUtensorMap* tm, uint64_t* bar) {
@@ -253,27 +265,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
       int terms_issued = 0;
       int slot = 0, ph = 1;  // empty-barrier phase: the first lap does not wait
       bool ok = true;
-      // a unit: two pieces.  as_n: B of S / dP (this CTA's 64 rows, both halves of the
-      // head dim); else B of the output GEMM (all 128 rows, this CTA's head-dim half)
+      // a unit.  as_n: B of S / dP (this CTA's 64 rows, the whole head dim, block c its
+      // columns 64c); else B of the output GEMM (all 128 rows, this CTA's head-dim half,
+      // blocks 2p, 2p + 1 the two 64-column blocks of rows 64p)
       auto load_unit = [&](const CUtensorMap* tm, int t, bool as_n) {
         const int hd = kind == kDQ ? it.kvh : it.h_base + t / it.nst;
         const int r0 = (it.lo + (kind == kDQ ? t : t % it.nst)) * BN;
-#pragma unroll 1
-        for (int p = 0; p < 2 && ok; ++p) {
-          if (!mbar_wait(&sm.empty[slot], ph, abort, P.status)) {
-            ok = false;
-            return;
-          }
-          if (rank == 0) mbar_arrive_expect_tx(&sm.full[slot], 2 * PR * PC * 2);
-          const uint32_t lb = lead_addr(&sm.full[slot]);
-          bf16* dst = ring0 + slot * (PR * PC);
-          const int row = as_n ? r0 + rank * PR : r0 + p * PR, col = as_n ? p * PC : rank * PC;
-          tma_load_pair(dst, tm, lb, col, hd, bstr, row, it.b);
-          tma_load_pair(dst + PR * 64, tm, lb, col + 64, hd, bstr, row, it.b);
-          if (++slot == nslot) {
-            slot = 0;
-            ph ^= 1;
-          }
+        if (!mbar_wait(&sm.empty[slot], ph, abort, P.status)) {
+          ok = false;
+          return;
+        }
+        if (rank == 0) mbar_arrive_expect_tx(&sm.full[slot], 2 * SLOT * 2);
+        const uint32_t lb = lead_addr(&sm.full[slot]);
+        bf16* dst = ring0 + slot * SLOT;
+        for (int c = 0; c < 4; ++c) {
+          const int row = as_n ? r0 + rank * PR : r0 + (c >> 1) * PR;
+          const int col = as_n ? c * 64 : rank * PC + (c & 1) * 64;
+          tma_load_pair(dst + c * PR * 64, tm, lb, col, hd, bstr, row, it.b);
+        }
+        if (++slot == nslot) {
+          slot = 0;
+          ph ^= 1;
         }
       };
       // the row terms of step t (DK, DV), into the buffer that step t-2 has read
@@ -318,15 +330,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
       constexpr uint32_t idO = idesc_bf16(2 * BM, DH, 0, 1);  // output: A in TMEM, B MN-major
       // descriptors encoded once; a block, slot or k-step adds its byte offset / 16
       const uint64_t a1d = sdesc_sw128(smem_u32(sm.a1), 16, 1024), a2d = sdesc_sw128(smem_u32(sm.a2), 16, 1024);
-      const uint64_t bK = sdesc_sw128(smem_u32(ring0), 16, 1024);          // pieces K-major
-      const uint64_t bM = sdesc_sw128(smem_u32(ring0), PR * 128, 1024);    // pieces MN-major
+      const uint64_t bK = sdesc_sw128(smem_u32(ring0), 16, 1024);        // slots K-major
+      const uint64_t bM = sdesc_sw128(smem_u32(ring0), PR * 128, 1024);  // slots MN-major
       int slot = 0, ph = 0;
       auto wait_w = [&](uint64_t* bar, int par) -> bool {
         if (!__all_sync(0xffffffffu, mbar_wait(bar, par & 1, abort, P.status))) return false;
         tc_fence_after();
         return true;
       };
-      auto next_piece = [&]() {
+      auto next_slot = [&]() {
         if (++slot == nslot) {
           slot = 0;
           ph ^= 1;
@@ -334,43 +346,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
       };
       // D[256 x 128] = A B^T over the head dim, then a signal that it is complete
       auto gemm_n = [&](uint32_t col, uint64_t ad, uint64_t* done) -> bool {
+        if (!wait_w(&sm.full[slot], ph)) return false;
+        const uint64_t bd = bK + (uint64_t)(slot * (SLOT * 2 / 16));
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-          if (!wait_w(&sm.full[slot], ph)) return false;
-          const uint64_t bd = bK + (uint64_t)(slot * (PR * PC * 2 / 16));
-#pragma unroll
-          for (int k8 = 0; k8 < 8; ++k8) {
-            const int kk = p * 8 + k8;
-            mma2_ss(tmem + col, ad + (uint64_t)((kk >> 2) * (BM * 128 / 16) + (kk & 3) * 2),
-                    bd + (uint64_t)((k8 >> 2) * (PR * 128 / 16) + (k8 & 3) * 2), idS, kk > 0 ? 1u : 0u);
-          }
-          if (p == 1) commit2(done);
-          commit2(&sm.empty[slot]);
-          next_piece();
-        }
+        for (int kk = 0; kk < DH / 16; ++kk)
+          mma2_ss(tmem + col, ad + (uint64_t)((kk >> 2) * (BM * 128 / 16) + (kk & 3) * 2),
+                  bd + (uint64_t)((kk >> 2) * (PR * 128 / 16) + (kk & 3) * 2), idS, kk > 0 ? 1u : 0u);
+        commit2(done);
+        commit2(&sm.empty[slot]);
+        next_slot();
         return true;
       };
-      // out[256 x 256] += A[tmem] B over the 128 streamed rows.  The pieces are waited for
-      // before A (each wait costs about 100 cycles of a chain that ends with A).
+      // out[256 x 256] += A[tmem] B over the 128 streamed rows.  B is waited for before A
+      // (each wait costs about 100 cycles of a chain that ends with A).
       auto gemm_out = [&](uint32_t acol, uint64_t* a_full, int a_par, bool acc0) -> bool {
-        const int s0 = slot;
-        if (!wait_w(&sm.full[slot], ph)) return false;
-        next_piece();
-        const int s1 = slot;
         if (!wait_w(&sm.full[slot], ph) || !wait_w(a_full, a_par)) return false;
-        next_piece();
+        const uint64_t bd = bM + (uint64_t)(slot * (SLOT * 2 / 16));
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-          const uint64_t bd = bM + (uint64_t)((p ? s1 : s0) * (PR * PC * 2 / 16));
-#pragma unroll
-          for (int k4 = 0; k4 < 4; ++k4) {
-            const int kk = p * 4 + k4;
-            // P / dS: each 64-column half packed at the start of its own columns
-            mma2_ts(tmem + COL_OUT, tmem + acol + p * HB + k4 * 8, bd + (uint64_t)(k4 * 16 * 128 / 16), idO,
-                    (acc0 || kk > 0) ? 1u : 0u);
-          }
-          commit2(&sm.empty[p ? s1 : s0]);
-        }
+        for (int kk = 0; kk < BN / 16; ++kk)
+          // P / dS: each 64-column half packed at the start of its own columns
+          mma2_ts(tmem + COL_OUT, tmem + acol + (kk >> 2) * HB + (kk & 3) * 8,
+                  bd + (uint64_t)((kk >> 2) * (PR * PC * 2 / 16) + (kk & 3) * 16 * 128 / 16), idO,
+                  (acc0 || kk > 0) ? 1u : 0u);
+        commit2(&sm.empty[slot]);
+        next_slot();
         return true;
       };
       bool ok = wait_w(&sm.a1_full, 0) && gemm_n(0, a1d, &sm.s_full[0]);
@@ -641,7 +640,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
   tc_fence_before();
   __syncthreads();
   cluster_sync();  // neither CTA's barriers or TMEM are used any more
-  if (warp == 0) {
+  if (warp == 1) {
     tc_fence_after();
     tmem_dealloc_pair(tmem, 512);
   }
@@ -688,8 +687,8 @@ static long long key_items(const SfaGeom& g) {
 // Query-head chunks of the DK and DV items: the count with the least estimated time over
 // the chip's 76 CTA pairs, as the larger of a pair's share of all items and the longest
 // item (DK of the key pair with the most query tiles), plus the finalize pass where there
-// are chunks.  In units of 1000 cycles, measured at L = 4096: a step of DK, DV and DQ 4.1,
-// 2.5 and 3.8, an item's fixed part 10, the finalize pass 8 and its traffic (8 bytes
+// are chunks.  In units of 1000 cycles, measured at L = 4096: a step of DK, DV and DQ 3.6,
+// 2.1 and 3.1, an item's fixed part 10, the finalize pass 8 and its traffic (8 bytes
 // written and read per element and chunk at about 3.4 KB per cycle).  `room`: slices of
 // partial sums there is space for.  (One chunk too many costs little on long items, but
 // three sequences of 98 positions, fwd + bwd: 63 us with 12 chunks, two waves of short items, 50 us with 4.)
@@ -713,14 +712,14 @@ static int head_chunks(const SfaGeom& g, long long room, long long ndq) {
   }
   const double per = (double)items / npair;  // items of one key pair
   // DQ: as many row-tile products as DK, two row tiles to an item
-  const double dq = ndq * 10.0 + 3.8 * sum * per * grp;
+  const double dq = ndq * 10.0 + 3.1 * sum * per * grp;
   int best = 1;
   double best_cost = 0;
   for (int hs = 1; hs <= grp && hs <= room; ++hs) {
     const int hper = (grp + hs - 1) / hs;
     if ((grp + hper - 1) / hper != hs) continue;  // another count gives the same chunks
-    const double total = dq + 2.0 * items * hs * 10.0 + 6.6 * sum * per * grp;
-    const double longest = 10.0 + 4.1 * hper * most;
+    const double total = dq + 2.0 * items * hs * 10.0 + 5.7 * sum * per * grp;
+    const double longest = 10.0 + 3.6 * hper * most;
     const double share = total / kPairs;
     double cost = share > longest ? share : longest;
     if (hs > 1) cost += 8.0 + 16.0 * hs * g.B * g.q_ns * (double)g.Lv * g.Hkv * DH / 3.4e6;
@@ -764,6 +763,15 @@ cudaError_t launch_sfa_bwd_main_tc256(const void* q, const void* k, const void* 
   const int rows = p.head_pairs ? BM : 2 * BM, nh = p.head_pairs ? g.Hq / 2 : g.Hq;
   const long long ndq = (long long)((g.Lq + rows - 1) / rows) * nh * g.q_ns * g.B;
   p.hchunks = head_chunks(g, room, ndq);
+  p.grp = g.Hq / g.Hkv;
+  p.hper = (p.grp + p.hchunks - 1) / p.hchunks;
+  p.d_tile = make_fast_div((uint32_t)(p.hchunks * g.Hkv * g.q_ns * g.B));
+  p.d_hc = make_fast_div((uint32_t)p.hchunks);
+  p.d_kns = make_fast_div((uint32_t)(g.Hkv * g.q_ns));
+  p.d_rank = make_fast_div((uint32_t)(nh * g.q_ns * g.B));
+  p.d_hns = make_fast_div((uint32_t)(nh * g.q_ns));
+  p.d_ns = make_fast_div((uint32_t)g.q_ns);
+  p.d_grp = make_fast_div((uint32_t)p.grp);
   if (p.hchunks > 1 && p.dkv == nullptr) return cudaErrorInvalidValue;
   p.g = g;
   p.scale = scale;
