@@ -95,21 +95,6 @@ HD_DEVINLINE void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t
       : "memory");
 }
 
-// Tiled reduce-add shared -> global through a tensor map (fp32 add); elements
-// outside the tensor are skipped.  Tracked by the issuing thread's bulk group.
-HD_DEVINLINE void tma_reduce_add_5d(const CUtensorMap* m, const void* src, int c0, int c1, int c2, int c3,
-                                    int c4) {
-  asm volatile(
-      "cp.reduce.async.bulk.tensor.5d.global.shared::cta.add.tile.bulk_group"
-      " [%0, {%2, %3, %4, %5, %6}], [%1];\n" ::"l"(reinterpret_cast<uint64_t>(m)),
-      "r"(smem_u32(src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
-      : "memory");
-}
-HD_DEVINLINE void bulk_commit() { asm volatile("cp.async.bulk.commit_group;\n" ::: "memory"); }
-HD_DEVINLINE void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
-HD_DEVINLINE void bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory"); }
-HD_DEVINLINE void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
-
 // ---------------------------------------------------------------- tcgen05
 HD_DEVINLINE void tmem_alloc(uint32_t* dst, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(dst)),
@@ -126,36 +111,14 @@ HD_DEVINLINE void tc_fence_before() { asm volatile("tcgen05.fence::before_thread
 HD_DEVINLINE void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 HD_DEVINLINE void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
-// Arrive on `bar` once every tcgen05 operation this thread issued so far has completed.
-HD_DEVINLINE void tc_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                   smem_u32(bar))
-               : "memory");
-}
-
-// D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate.
-// No "memory" clobber: as a compiler memory barrier it cost the issuing thread
-// about 50 extra cycles per MMA.  Ordering against the shared-memory producers and
-// the TMEM readers comes from the mbarrier waits, tcgen05 fences and commits,
-// which are volatile asm statements with memory clobbers issued around these.
-HD_DEVINLINE void tc_mma_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum));
-}
-
-// D[tmem] (+)= A[tmem] * B[smem]: A (M x K, bf16 pairs packed per 32-bit column,
-// one row per TMEM lane) read from tensor memory.
-HD_DEVINLINE void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accum));
-}
-
-// Warp-collective forms: the whole warp runs the issue loop (warp-uniform control flow
-// and operands) and one lane chosen by elect.sync issues the instruction.
+// D[tmem] (+)= A * B, bf16 inputs, fp32 accumulate; B from shared memory, A from shared
+// memory (ss) or tensor memory (ts: M x K, bf16 pairs packed per 32-bit column, one row per
+// TMEM lane).  The whole warp runs the issue loop (warp-uniform control flow and operands)
+// and one lane chosen by elect.sync issues the instruction.  No "memory" clobber: as a
+// compiler memory barrier it cost the issuing thread about 50 extra cycles per MMA.
+// Ordering against the shared-memory producers and the TMEM readers comes from the
+// mbarrier waits, tcgen05 fences and commits, which are volatile asm statements with
+// memory clobbers issued around these.
 HD_DEVINLINE void tc_mma_ss_w(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
   asm volatile(
       "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n elect.sync _|e, 0xffffffff;\n"
@@ -168,6 +131,7 @@ HD_DEVINLINE void tc_mma_ts_w(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, 
       " @e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
       "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accum));
 }
+// Arrive on `bar` once every tcgen05 operation issued so far has completed.
 HD_DEVINLINE void tc_commit_w(uint64_t* bar) {
   asm volatile(
       "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
@@ -186,13 +150,6 @@ HD_DEVINLINE float ex2_approx(float x) {
 HD_DEVINLINE uint32_t cvt_bf16x2(float lo, float hi) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;\n" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
-}
-
-// Packed bf16 pair product, round to nearest even.
-HD_DEVINLINE uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
-  uint32_t r;
-  asm("mul.rn.bf16x2 %0, %1, %2;\n" : "=r"(r) : "r"(a), "r"(b));
   return r;
 }
 
@@ -228,11 +185,6 @@ HD_DEVINLINE void tmem_ld16(uint32_t taddr, uint32_t* r) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
-}
-HD_DEVINLINE void tmem_ld8(uint32_t taddr, uint32_t* r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
 }
 HD_DEVINLINE void tmem_st8(uint32_t taddr, const uint32_t* r) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"r"(taddr), "r"(r[0]),
@@ -296,12 +248,10 @@ HD_DEVINLINE void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;\
 HD_DEVINLINE void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
 
 // ---------------------------------------------------------------- host: tensor maps
-// Tensor map over a [B][nL][H][Dh] tensor (element size esize) seen as the 5-D array
+// Tensor map over a bf16 [B][nL][H][Dh] tensor seen as the 5-D array
 // {Dh, H, ns, Lv, B} (innermost first): virtual row r of stream s is position
-// r*rs + s.  Box = box_d elements x box_rows rows; swizzle128 selects the
-// 128-byte swizzle (box_d * esize must then be 128).  Defined in tmap.cu.
-bool make_rows_tmap(CUtensorMap* m, const void* base, const SfaGeom& g, int H, int Dh, int box_rows,
-                    int esize = 2, int box_d = 64, bool swizzle128 = true);
+// r*rs + s.  Box = 64 columns x box_rows rows, 128-byte swizzle.  Defined in tmap.cu.
+bool make_rows_tmap(CUtensorMap* m, const void* base, const SfaGeom& g, int H, int Dh, int box_rows);
 
 // ---------------------------------------------------------------- CTA pairs (cta_group::2)
 HD_DEVINLINE void tmem_alloc_pair(uint32_t* dst, uint32_t ncols) {
