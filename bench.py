@@ -4,9 +4,7 @@
 One step = one pass of the hot path over one synthetic batch of the
 Qwen3-8B-class layer (B=1, L=4096 tokens, n=4 -> 16384 positions, Hq=32, Hkv=8,
 Dh=128, bf16, intra-stream / WITHIN mask):
-  expansion gather (4 tables of 151936 x 4096)  -> sfa_fwd -> sfa_bwd_row_terms
-  -> sfa_bwd_main -> sfa_bwd_finalize, with sfa_bwd_clear on a side stream beside
-  the forward.
+  expansion gather (4 tables of 151936 x 4096)  -> sfa_fwd -> sfa_bwd.
 Metric: attention FLOPs over visible pairs only (forward 4*Dh, backward 10*Dh per
 pair and query head) per second of the whole step, in TFLOP/s.
 
@@ -166,7 +164,7 @@ class ClockSampler:
 
 # ---------------------------------------------------------------- the step
 class HotPath:
-    """Device buffers and the five launches of one step."""
+    """Device buffers and the calls of one step."""
 
     def __init__(self, s: AttnShape, mode: int, dev, with_gather: bool = True, seed: int = 1, window: int = 0):
         from paper_2607_08186_gb300 import binding
@@ -194,11 +192,8 @@ class HotPath:
             self.x = torch.empty(s.B, s.nL, GATHER_D, dtype=torch.bfloat16, device=dev)
         self.host_out = [torch.empty(t.shape, dtype=t.dtype, pin_memory=True)
                          for t in (self.o, self.lse, self.dq, self.dk, self.dv)]
-        # the dQ accumulator is cleared on a side stream beside the forward (it needs
-        # nothing from it), after the previous step's finalize has read it
-        self.side = torch.cuda.Stream(device=dev)
-        self.ev_start, self.ev_clear, self.ev_fin = torch.cuda.Event(), torch.cuda.Event(), torch.cuda.Event()
-        self.launches_per_step = 5 + (1 if with_gather else 0)
+        # forward; row terms and the main pass of the backward; gather
+        self.launches_per_step = 3 + (1 if with_gather else 0)
 
     def _bufs(self):
         return {"q": self.q, "k": self.k, "v": self.v, "do": self.do, "ids": getattr(self, "ids", None),
@@ -207,14 +202,6 @@ class HotPath:
     def step(self, ev=None, bufs=None, stream=None):
         b, s = self.b, self.s
         t = bufs or self._bufs()
-        main = stream if stream is not None else torch.cuda.current_stream()
-        # the side stream's clear starts only once this step has started on the main
-        # stream (so it is inside a timed step) and the previous step's dQ is out
-        self.ev_start.record(main)
-        self.side.wait_event(self.ev_start)
-        self.side.wait_event(self.ev_fin)
-        b.sfa_bwd_clear(s.B, s.L, s.n, s.Hq, s.Hkv, s.Dh, self.mode, self.ws, stream=self.side)
-        self.ev_clear.record(self.side)
         if self.with_gather:
             b.hd_expand_embed(self.tables, t["ids"], self.x, stream=stream)
         if ev is not None:
@@ -222,20 +209,14 @@ class HotPath:
         b.sfa_fwd(t["q"], t["k"], t["v"], t["o"], t["lse"], s.n, self.mode, window=self.window, stream=stream)
         if ev is not None:
             ev[1].record()
-        b.sfa_bwd_row_terms(t["o"], t["do"], t["lse"], s.n, self.mode, self.ws, s.Hkv, stream=stream)
-        main.wait_event(self.ev_clear)
+        b.sfa_bwd(t["q"], t["k"], t["v"], t["o"], t["lse"], t["do"], t["dq"], t["dk"], t["dv"], s.n, self.mode,
+                  self.ws, window=self.window, stream=stream)
         if ev is not None:
             ev[2].record()
-        b.sfa_bwd_main(t["q"], t["k"], t["v"], t["do"], t["dk"], t["dv"], s.n, self.mode, self.ws,
-                       window=self.window, stream=stream)
-        if ev is not None:
-            ev[3].record()
-        b.sfa_bwd_finalize(t["dq"], s.n, self.mode, self.ws, s.Hkv, stream=stream)
-        self.ev_fin.record(main)
 
     def e2e(self, steps: int, warmup: int, ws: int) -> float:
         """Seconds per step end to end with host buffers: every step copies its inputs
-        host -> device (pinned), runs the five launches and copies its results device ->
+        host -> device (pinned), runs the step and copies its results device ->
         host.  Three streams overlap step k+1's upload and step k-1's download with step
         k's compute; two device buffer sets, ordered by events, keep them apart."""
         sets = [self._bufs()]
@@ -296,7 +277,7 @@ class L2Flush:
         self.buf.zero_()
 
 
-def timed_steps(step, iters: int, warmup: int, flush: L2Flush, ws: int = 1, nev: int = 4):
+def timed_steps(step, iters: int, warmup: int, flush: L2Flush, ws: int = 1, nev: int = 3):
     """Median device time (s) of `iters` calls of step(ev): each call bracketed by its own
     CUDA events on the launching stream, the L2 flushed between calls outside the events,
     `warmup` untimed calls first; ev holds `nev` events the step may record inside.
@@ -320,16 +301,16 @@ def timed_steps(step, iters: int, warmup: int, flush: L2Flush, ws: int = 1, nev:
 
 
 def measure_layer(s: AttnShape, mode: int, dev, iters=10, warmup=3, window: int = 0, flush=None):
-    """fwd, bwd-main and fwd+bwd times of one layer (no gather), seconds: medians over
+    """fwd, bwd and fwd+bwd times of one layer (no gather), seconds: medians over
     `iters` steps with the L2 flushed between them."""
     hp = HotPath(s, mode, dev, with_gather=False, seed=7, window=window)
     flush = flush or L2Flush(dev)
     total, evs = timed_steps(lambda ev: hp.step(ev), iters, warmup, flush)
     fwd = statistics.median(e[0].elapsed_time(e[1]) for e in evs) / 1e3
-    bwd = statistics.median(e[2].elapsed_time(e[3]) for e in evs) / 1e3
+    bwd = statistics.median(e[1].elapsed_time(e[2]) for e in evs) / 1e3
     del hp
     torch.cuda.empty_cache()
-    return {"fwd_s": fwd, "bwd_main_s": bwd, "step_s": total}
+    return {"fwd_s": fwd, "bwd_s": bwd, "step_s": total}
 
 
 # ---------------------------------------------------------------- bandwidth ops
@@ -476,7 +457,7 @@ def measure_moe_stack(dev, pk, steps: int = 3, warmup: int = 1):
     del layers
     torch.cuda.empty_cache()
     return {"workload": "moe_large_n4 stack: B=1 L=8192 n=4 (32768 positions) Hq=64 Hkv=8 Dh=128, "
-                        "7 WITHIN + 1 CROSS layers, fwd+bwd (prep, main, finalize) per layer",
+                        "7 WITHIN + 1 CROSS layers, fwd+bwd per layer",
             "ms_per_stack": sec * 1e3, "flops_per_stack": flops, "tflops": flops / sec / 1e12,
             "frac": flops / sec / 1e12 / pk["bf16"], "frac_of_sustained": flops / sec / 1e12 / pk["bf16_sustained"],
             "within_layer_ms": within_ms, "within_layer_tflops": attn_flops(s, WITHIN, 14) / within_ms / 1e9,
@@ -587,10 +568,10 @@ def measure_decode(dev, hbm_peak: float, quick: bool = False):
 
 
 # ---------------------------------------------------------------- ncu traffic record
-# ABI phase -> (kernel symbol, source file) of the implementation the library runs.
+# ABI call -> (main kernel's symbol, source file) of the implementation the library runs.
 KERNEL_OF = {
     "sfa_fwd": ("hdsfa::tcfwd::fwd_kernel<128, false>", "sfa_fwd_tc.cu"),
-    "sfa_bwd_main": ("hdsfa::tcbwd::bwd_kernel<128, false>", "sfa_bwd_tc.cu"),
+    "sfa_bwd": ("hdsfa::tcbwd::bwd_kernel<128>", "sfa_bwd_tc.cu"),
 }
 
 
@@ -751,7 +732,7 @@ def main():
             print(json.dumps({"layer": f"{name}_{args.layer_only}", "ms": r["step_s"] * 1e3,
                               "tflops": fl / r["step_s"] / 1e12, "fwd_ms": r["fwd_s"] * 1e3,
                               "fwd_tflops": attn_flops(ls, mode, FWD_FLOP, w) / r["fwd_s"] / 1e12,
-                              "bwd_main_ms": r["bwd_main_s"] * 1e3}), flush=True)
+                              "bwd_ms": r["bwd_s"] * 1e3}), flush=True)
         return
     hp = HotPath(s, WITHIN, dev, with_gather=True, seed=1)
     flops_step = attn_flops(s, WITHIN, FWD_FLOP + BWD_FLOP)
@@ -771,11 +752,11 @@ def main():
     clk = clocks.stop()
     value, sec_max = job_throughput(flops_step, sec, ws)
     fwd_s = statistics.median(e[0].elapsed_time(e[1]) for e in evs) / 1e3
-    bwd_s = statistics.median(e[2].elapsed_time(e[3]) for e in evs) / 1e3
+    bwd_s = statistics.median(e[1].elapsed_time(e[2]) for e in evs) / 1e3
     bwd_flops = attn_flops(s, WITHIN, BWD_FLOP)
     fwd_flops = attn_flops(s, WITHIN, FWD_FLOP)
-    dom = "sfa_bwd_main" if bwd_s >= fwd_s else "sfa_fwd"
-    dom_flops, dom_s = (bwd_flops, bwd_s) if dom == "sfa_bwd_main" else (fwd_flops, fwd_s)
+    dom = "sfa_bwd" if bwd_s >= fwd_s else "sfa_fwd"
+    dom_flops, dom_s = (bwd_flops, bwd_s) if dom == "sfa_bwd" else (fwd_flops, fwd_s)
     achieved = dom_flops / dom_s / 1e12
     tr = traffic_record(dom)
 
@@ -810,7 +791,7 @@ def main():
                      "frac_of_sustained": achieved / pk["bf16_sustained"],
                      "peak_source": f"{pk['src']} bf16 dense burst", "traffic": tr,
                      "algorithmic_flops_per_launch": dom_flops, "avg_launch_ms": dom_s * 1e3},
-        "kernels_ms": {"sfa_fwd": fwd_s * 1e3, "sfa_bwd_main": bwd_s * 1e3},
+        "kernels_ms": {"sfa_fwd": fwd_s * 1e3, "sfa_bwd": bwd_s * 1e3},
         "e2e": {"value": e2e_val / 1e12, "unit": "TFLOP/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "ms_per_step": e2e_s * 1e3},
         "gpu_launches": launches,
@@ -822,7 +803,7 @@ def main():
         fl = attn_flops(s, CROSS, FWD_FLOP + BWD_FLOP)
         extras["cross_layer"] = {"workload": f"{WORKLOAD}_cross", "tflops": fl / r["step_s"] / 1e12,
                                  "fwd_tflops": attn_flops(s, CROSS, FWD_FLOP) / r["fwd_s"] / 1e12,
-                                 "bwd_main_tflops": attn_flops(s, CROSS, BWD_FLOP) / r["bwd_main_s"] / 1e12,
+                                 "bwd_tflops": attn_flops(s, CROSS, BWD_FLOP) / r["bwd_s"] / 1e12,
                                  "ms": r["step_s"] * 1e3}
         sweep = []
         for n in (1, 2, 4, 8):
@@ -846,7 +827,7 @@ def main():
             fl = attn_flops(s, LOCAL, FWD_FLOP + BWD_FLOP, w)
             loc.append({"window_positions": w, "ms": r["step_s"] * 1e3, "tflops": fl / r["step_s"] / 1e12,
                         "fwd_tflops": attn_flops(s, LOCAL, FWD_FLOP, w) / r["fwd_s"] / 1e12,
-                        "bwd_main_tflops": attn_flops(s, LOCAL, BWD_FLOP, w) / r["bwd_main_s"] / 1e12})
+                        "bwd_tflops": attn_flops(s, LOCAL, BWD_FLOP, w) / r["bwd_s"] / 1e12})
         extras["local_layer"] = {"workload": f"{WORKLOAD}_local", "windows": loc}
         # head dim 256 (80B-class heads: 24 query over 2 K/V heads): the head-dim-256
         # tcgen05 forward and backward kernels
@@ -857,7 +838,7 @@ def main():
             "workload": "B=1 L=4096 n=4 Hq=24 Hkv=2 Dh=256, WITHIN, fwd+bwd (head-dim-256 tcgen05 kernels)",
             "ms": r["step_s"] * 1e3, "tflops": fl / r["step_s"] / 1e12,
             "fwd_tflops": attn_flops(s80, WITHIN, FWD_FLOP) / r["fwd_s"] / 1e12,
-            "bwd_main_tflops": attn_flops(s80, WITHIN, BWD_FLOP) / r["bwd_main_s"] / 1e12}
+            "bwd_tflops": attn_flops(s80, WITHIN, BWD_FLOP) / r["bwd_s"] / 1e12}
         extras["expansion_backward"] = measure_expansion_backward(dev, pk["hbm"])
         extras["decode"] = measure_decode(dev, pk["hbm"], quick=True)
         extras["final_stream_layer"] = measure_final_layer(dev, pk["bf16"], flush=flush)
