@@ -45,6 +45,7 @@ __global__ void __launch_bounds__(256) sfa_bwd_prep_kernel(const bf16* __restric
   if ((long long)w >= (long long)g.B * ns * nrb * Hq) return;
   const unsigned h = w % Hq, w1 = w / Hq, rb = w1 % nrb, w2 = w1 / nrb, s = w2 % ns, b = w2 / ns;
   const unsigned r0 = rb * RPW;
+  attn_dep_wait(8);
   uint4 xo[ITER], xd[ITER];
 #pragma unroll
   for (int i = 0; i < ITER; ++i) {
@@ -124,23 +125,10 @@ cudaError_t launch_sfa_bwd_prep(const void* o, const void* dout, const float* ls
   const long long warps = (long long)g.B * g.ns * (row_terms_pitch(g.Lv) / 8) * g.Hq;  // 8 rows of one problem each
   const unsigned blocks = (unsigned)((warps * 32 + 255) / 256);
   const bf16 *ob = (const bf16*)o, *db = (const bf16*)dout;
-  if (Dh == 256) {
-    if (zero)
-      sfa_bwd_prep_kernel<256, true><<<blocks, 256, 0, st>>>(ob, db, lse, lse2_ws, delta_ws, dq_ws, g);
-    else
-      sfa_bwd_prep_kernel<256, false><<<blocks, 256, 0, st>>>(ob, db, lse, lse2_ws, delta_ws, dq_ws, g);
-  } else if (Dh == 64) {
-    if (zero)
-      sfa_bwd_prep_kernel<64, true><<<blocks, 256, 0, st>>>(ob, db, lse, lse2_ws, delta_ws, dq_ws, g);
-    else
-      sfa_bwd_prep_kernel<64, false><<<blocks, 256, 0, st>>>(ob, db, lse, lse2_ws, delta_ws, dq_ws, g);
-  } else {
-    if (zero)
-      sfa_bwd_prep_kernel<128, true><<<blocks, 256, 0, st>>>(ob, db, lse, lse2_ws, delta_ws, dq_ws, g);
-    else
-      sfa_bwd_prep_kernel<128, false><<<blocks, 256, 0, st>>>(ob, db, lse, lse2_ws, delta_ws, dq_ws, g);
-  }
-  return cudaGetLastError();
+  const auto kernel = Dh == 256 ? (zero ? sfa_bwd_prep_kernel<256, true> : sfa_bwd_prep_kernel<256, false>)
+                      : Dh == 64 ? (zero ? sfa_bwd_prep_kernel<64, true> : sfa_bwd_prep_kernel<64, false>)
+                                 : (zero ? sfa_bwd_prep_kernel<128, true> : sfa_bwd_prep_kernel<128, false>);
+  return launch_attn(kernel, blocks, 256, 0, st, ob, db, lse, lse2_ws, delta_ws, dq_ws, g);
 }
 
 cudaError_t launch_sfa_bwd_clear(float* dq_ws, const SfaGeom& g, int Dh, cudaStream_t st) {

@@ -195,6 +195,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) bwd_kernel(const __grid_constant_
     sm.abort = 0;
     fence_mbar_init();
   }
+  attn_dep_wait(1);
   const Item it = make_item(P, (int)blockIdx.x);
   const int kind = it.kind, T = it.T;
   const size_t half = (size_t)G.B * G.q_ns * G.Lv * G.Hkv * DH;  // elements of a slice half
@@ -727,6 +728,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) bwd_kernel(const __grid_constant_
 template <int DH>
 __global__ void __launch_bounds__(256) dkv_finalize_kernel(const float* __restrict__ dkv, bf16* __restrict__ dk,
                                                            bf16* __restrict__ dv, SfaGeom g, int chunks) {
+  attn_dep_wait(8);
   const long long n8 = (long long)g.B * g.q_ns * g.Lv * g.Hkv * (DH / 8);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n8) return;
@@ -809,12 +811,10 @@ static cudaError_t bwd_tc_impl(tcbwd::Params& p, long long slice, cudaStream_t s
   cudaError_t e = cudaFuncSetAttribute(bwd_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const long long ndq = (long long)((g.Lq + BM - 1) / BM) * g.Hq * g.q_ns * g.B;
-  bwd_kernel<DH><<<(unsigned)(p.nkv + ndq), NTHREADS, smem, st>>>(p);
-  e = cudaGetLastError();
+  e = launch_attn(bwd_kernel<DH>, p.nkv + ndq, NTHREADS, smem, st, p);
   if (e != cudaSuccess || p.hchunks == 1) return e;
   const long long n8 = slice / 8;
-  dkv_finalize_kernel<DH><<<(unsigned)((n8 + 255) / 256), 256, 0, st>>>(p.dkv, p.dk, p.dv, g, p.hchunks);
-  return cudaGetLastError();
+  return launch_attn(dkv_finalize_kernel<DH>, (n8 + 255) / 256, 256, 0, st, p.dkv, p.dk, p.dv, g, p.hchunks);
 }
 
 // Dh: 64 or 128.  dq_out: bf16 dQ (scaled); null: unscaled fp32 dQ into dq_ws.  With dq_out

@@ -185,6 +185,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
   const SfaGeom& G = P.g;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)(blockIdx.x & 1);  // = %cluster_ctarank
+  attn_dep_wait(1);
   const Item it = make_item(P, (int)(blockIdx.x >> 1), rank);
   const int kind = it.kind, T = it.T;
   const size_t half = (size_t)G.B * G.q_ns * G.Lv * G.Hkv * DH;  // elements of a slice half
@@ -649,6 +650,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
 // order, 8 columns per thread.
 __global__ void __launch_bounds__(256) dkv_finalize_kernel(const float* __restrict__ dkv, bf16* __restrict__ dk,
                                                            bf16* __restrict__ dv, SfaGeom g, int chunks) {
+  attn_dep_wait(8);
   const long long n8 = (long long)g.B * g.q_ns * g.Lv * g.Hkv * (DH / 8);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n8) return;
@@ -781,12 +783,10 @@ cudaError_t launch_sfa_bwd_main_tc256(const void* q, const void* k, const void* 
   const long long grid = 2 * (2LL * p.nkv + ndq);
   cudaError_t e = cudaFuncSetAttribute(bwd256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   if (e != cudaSuccess) return e;
-  bwd256_kernel<<<(unsigned)grid, NTHREADS, kSmemBytes, st>>>(p);
-  e = cudaGetLastError();
+  e = launch_attn(bwd256_kernel, grid, NTHREADS, kSmemBytes, st, p);
   if (e != cudaSuccess || p.hchunks == 1) return e;
   const long long n8 = slice / 8;
-  dkv_finalize_kernel<<<(unsigned)((n8 + 255) / 256), 256, 0, st>>>(p.dkv, (bf16*)dk, (bf16*)dv, g, p.hchunks);
-  return cudaGetLastError();
+  return launch_attn(dkv_finalize_kernel, (n8 + 255) / 256, 256, 0, st, p.dkv, (bf16*)dk, (bf16*)dv, g, p.hchunks);
 }
 
 }  // namespace hdsfa

@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
     tmem_relinquish();
     tc_fence_before();
   }
+  attn_dep_wait(1);
   // A CTA's two query tiles: with head_pairs the same 128 rows of heads 2x and 2x+1
   // (one K/V group: both tiles see exactly the same key tiles and finish together),
   // else rows m0 and m0 + 128 of one head (the second tile sees one more key tile).
@@ -469,8 +470,7 @@ static cudaError_t tc_fwd_impl(tcfwd::Params& p, cudaStream_t st) {
   const int rows_per_cta = p.head_pairs ? tcfwd::BM : tcfwd::NG * tcfwd::BM;
   const int nh = p.head_pairs ? p.g.Hq / tcfwd::NG : p.g.Hq;
   const unsigned grid = (unsigned)((p.g.Lq + rows_per_cta - 1) / rows_per_cta) * (unsigned)(nh * p.g.q_ns * p.g.B);
-  tcfwd::fwd_kernel<DH, NAIVE><<<grid, tcfwd::NTHREADS, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_attn(tcfwd::fwd_kernel<DH, NAIVE>, grid, tcfwd::NTHREADS, smem, st, p);
 }
 
 cudaError_t launch_sfa_fwd_tc(const void* q, const void* k, const void* v, void* o, float* lse,

@@ -110,6 +110,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) fwd256_
     tmem_alloc_pair(&sm.tmem_base, 512);
     tc_fence_before();
   }
+  attn_dep_wait(1);
   // linear grid of pairs, query-tile rank slowest: the last query tiles (the most key tiles
   // to visit) of every head, stream and batch launch first
   const int hp = P.head_pairs, rows = hp ? BM : 2 * BM, nh = hp ? G.Hq / 2 : G.Hq;
@@ -426,8 +427,7 @@ cudaError_t launch_sfa_fwd_tc256(const void* q, const void* k, const void* v, vo
   cudaError_t e = cudaFuncSetAttribute(fwd256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
   if (e != cudaSuccess) return e;
   const unsigned grid = 2 * (unsigned)((g.Lq + rows - 1) / rows) * (unsigned)(nh * g.q_ns * g.B);
-  fwd256_kernel<<<grid, NTHREADS, kSmemBytes, st>>>(p);
-  return cudaGetLastError();
+  return launch_attn(fwd256_kernel, grid, NTHREADS, kSmemBytes, st, p);
 }
 
 }  // namespace hdsfa
