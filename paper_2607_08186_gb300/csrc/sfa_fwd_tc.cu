@@ -164,6 +164,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
   int lo[NG], hi[NG];
 #pragma unroll
   for (int g = 0; g < NG; ++g) tile_range(G, qm[g], lo[g], hi[g]);
+  // The window of a final-stream problem whose query step is wider than it can leave key
+  // tiles between the two query tiles' ranges that neither of them sees.  Tiles are numbered
+  // without that gap (the second tile's lie `gap` further on), so some group takes part at
+  // every j: its softmax waits for the tiles on the issuer's behalf, its PV releases K(j).
+  static_assert(NG == 2, "one gap");
+  const int gap = hi[1] >= lo[1] ? max(0, lo[1] - hi[0] - 1) : 0;
+  lo[1] -= gap;
+  hi[1] -= gap;
   const int n_lo = lo[0];
   int n_hi = hi[0];
 #pragma unroll
@@ -190,8 +198,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
           return;
         }
         mbar_arrive_expect_tx(&sm.full[slot], BN * DH * 2);
+        const int row = (j > hi[0] ? j + gap : j) * BN;
         for (int c = 0; c < DH / 64; ++c)
-          tma_load_5d(sm.ring[slot] + c * BN * 64, tm, &sm.full[slot], c * 64, kvh, sk, j * BN, b);
+          tma_load_5d(sm.ring[slot] + c * BN * 64, tm, &sm.full[slot], c * 64, kvh, sk, row, b);
         ++issued;
         if (++slot == NSLOT) {
           slot = 0;
@@ -306,6 +315,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
     bool ok = true;
     for (int j = lo[g]; j <= hi[g]; ++j) {
       const int i = j - lo[g];
+      const int kb = (g == 0 ? j : j + gap) * BN;  // first key row of the tile
       // this thread's arrivals on p_full also say that V(j) and K(j+1) have landed (waited
       // for here, where the softmax waits for S anyway)
       if (warp == 2 + 4 * g && lane == 0) {
@@ -326,26 +336,26 @@ __global__ void __launch_bounds__(NTHREADS, 1) fwd_kernel(const __grid_constant_
       tmem_ld_wait();
       // tiles holding a key past the first query's key row (the diagonal band), a key at
       // or below the last query's window edge, and the ragged last tile
-      const bool need_mask = (j + 1) * BN - 1 > rq0 || (G.window > 0 && j * BN <= rq1 - G.window) ||
-                             (j + 1) * BN > G.Lv;
+      const bool need_mask = kb + BN - 1 > rq0 || (G.window > 0 && kb <= rq1 - G.window) ||
+                             kb + BN > G.Lv;
       if constexpr (NAIVE) {
         // causal (no window in this schedule) and k = (rq - key row) mod smod == 0,
         // k stepped down the tile's columns
-        int k = (rq - j * BN) % G.smod;
+        int k = (rq - kb) % G.smod;
         if (k < 0) k += G.smod;
 #pragma unroll
         for (int e = 0; e < BN; ++e) {
-          if (k != 0 || j * BN + e > rq || j * BN + e >= G.Lv) x[e] = -INFINITY;
+          if (k != 0 || kb + e > rq || kb + e >= G.Lv) x[e] = -INFINITY;
           k = k == 0 ? G.smod - 1 : k - 1;
         }
       } else if (need_mask) {
         // keys past the query's own row or the end, and (LOCAL) at or below its window edge
-        const int e_hi = min(rq, G.Lv - 1) - j * BN;
+        const int e_hi = min(rq, G.Lv - 1) - kb;
 #pragma unroll
         for (int e = 0; e < BN; ++e)
           if (e > e_hi) x[e] = -INFINITY;
         if (G.window > 0) {
-          const int e_lo = rq - G.window + 1 - j * BN;
+          const int e_lo = rq - G.window + 1 - kb;
 #pragma unroll
           for (int e = 0; e < BN; ++e)
             if (e < e_lo) x[e] = -INFINITY;
