@@ -77,7 +77,9 @@ hd_status_t make_geom(int B, int L, int n, int Hq, int Hkv, int Dh, sfa_mode_t m
     g->Lv = (int)nL;
     g->ns = 1;
     g->rs = 1;
-    g->window = mode == SFA_LOCAL ? window : 0;
+    // a window of nL positions already sees every earlier key; larger ones ("no limit",
+    // up to INT_MAX) are cut to it, so that sums of a row and the window stay in 32 bits
+    g->window = mode == SFA_LOCAL ? (window < nL ? window : (int)nL) : 0;
   }
   g->smod = mode == SFA_WITHIN_NAIVE ? n : 0;
   // queries are the key rows themselves
