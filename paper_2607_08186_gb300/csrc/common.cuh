@@ -143,6 +143,10 @@ HD_DEVINLINE int swz(int row, int col) {
 // kernel before it in the stream is finishing.  It waits (grid_dep_wait) for that kernel's
 // completion before it touches global memory, and lets its own successor start its set-up
 // (grid_dep_launch).  Without the launch attribute both are no-ops.
+// Such a kernel overlaps the one that writes its inputs, so it reads them with plain loads:
+// the read-only path (__ldg, or a const __restrict__ pointer, from which the compiler takes
+// it) is for data nobody writes while the kernel runs, and its loads may be moved above the
+// wait.
 HD_DEVINLINE void grid_dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 HD_DEVINLINE void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 

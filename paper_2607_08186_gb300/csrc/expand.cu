@@ -1,16 +1,14 @@
 // Multi-stream token expansion (Eq. 1): out[b][t*n + s][:] = tables[s][ids[b][t]][:].
 //
 // HBM-bound bit copy.  One warp per output row (b, t, s): it reads the table row
-// with 16-byte non-coherent loads (the tables are read-only during the kernel) and
-// writes the contiguous output row with 16-byte stores, four vectors in flight per
-// lane.  Output rows are visited in memory order, so consecutive warps write
+// with 16-byte loads and writes the contiguous output row with 16-byte stores, four
+// vectors in flight per lane.  Output rows are visited in memory order, so consecutive warps write
 // consecutive rows.
 #include "common.cuh"
 
 namespace hdsfa {
 
-__global__ void __launch_bounds__(256) expand_embed_kernel(const uint4* __restrict__ tables,
-                                                           const int32_t* __restrict__ ids,
+__global__ void __launch_bounds__(256) expand_embed_kernel(const uint4* tables, const int32_t* ids,
                                                            uint4* __restrict__ out, long long rows,
                                                            int n, int V, int D16, int32_t* status) {
   const int lane = threadIdx.x & 31;
@@ -20,7 +18,7 @@ __global__ void __launch_bounds__(256) expand_embed_kernel(const uint4* __restri
   grid_dep_launch();
   for (long long row = warp0; row < rows; row += nwarps) {
     const int s = (int)(row % n);
-    const int id = __ldg(ids + row / n);
+    const int id = ids[row / n];
     uint4* dst = out + row * D16;
     if (id < 0 || id >= V) {
       for (int c = lane; c < D16; c += 32) dst[c] = make_uint4(0, 0, 0, 0);
@@ -30,14 +28,13 @@ __global__ void __launch_bounds__(256) expand_embed_kernel(const uint4* __restri
     const uint4* src = tables + ((long long)s * V + id) * D16;
     int c = lane;
     for (; c + 96 < D16; c += 128) {
-      uint4 a0 = __ldg(src + c), a1 = __ldg(src + c + 32), a2 = __ldg(src + c + 64),
-            a3 = __ldg(src + c + 96);
+      const uint4 a0 = src[c], a1 = src[c + 32], a2 = src[c + 64], a3 = src[c + 96];
       dst[c] = a0;
       dst[c + 32] = a1;
       dst[c + 64] = a2;
       dst[c + 96] = a3;
     }
-    for (; c < D16; c += 32) dst[c] = __ldg(src + c);
+    for (; c < D16; c += 32) dst[c] = src[c];
   }
 }
 

@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kSortThreads) chunk_kernel(unsigned long long*
 // for the first key of an id (no key of its id below it), appends the id's run
 // record.  Block (0, 0) also clears the run counters.
 constexpr int kField = 21;
-__global__ void __launch_bounds__(kRankTile) rank_kernel(const int32_t* __restrict__ ids, long long N, int V,
+__global__ void __launch_bounds__(kRankTile) rank_kernel(const int32_t* ids, long long N, int V,
                                                         unsigned long long* __restrict__ partial,
                                                         unsigned* __restrict__ counts, int32_t* status) {
   // Ids in 32 bits; outside the diagonal tiles the order of the tokens is the tiles', so a
@@ -142,8 +142,8 @@ __global__ void __launch_bounds__(kRankTile) rank_kernel(const int32_t* __restri
                                 ((unsigned long long)same_below << (2 * kField));
 }
 
-__global__ void __launch_bounds__(256) scatter_kernel(const int32_t* __restrict__ ids, long long N, int V,
-                                                      const unsigned long long* __restrict__ partial, int tiles,
+__global__ void __launch_bounds__(256) scatter_kernel(const int32_t* ids, long long N, int V,
+                                                      const unsigned long long* partial, int tiles,
                                                       unsigned long long* __restrict__ keys, uint4* __restrict__ light,
                                                       uint4* __restrict__ heavy, unsigned* __restrict__ counts) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -241,12 +241,9 @@ HD_DEVINLINE void rmw_add(float* dst, const float4& a0, const float4& a1, const 
 //   heavy: warp w sums the chunk over the w-th of kHeavyBlocks consecutive token
 //          blocks; warp 0 adds the block sums in block order.
 // Every element of dE is read and written by exactly one thread.
-__global__ void __launch_bounds__(kRowThreads, 3) rows_kernel(const bf16* __restrict__ dx,
-                                                          const unsigned long long* __restrict__ keys,
-                                                          const uint4* __restrict__ light,
-                                                          const uint4* __restrict__ heavy,
-                                                          const unsigned* __restrict__ counts,
-                                                          float* __restrict__ de, long long N, int n, int V,
+__global__ void __launch_bounds__(kRowThreads, 3) rows_kernel(const bf16* dx, const unsigned long long* keys,
+                                                          const uint4* light, const uint4* heavy,
+                                                          const unsigned* counts, float* __restrict__ de, long long N, int n, int V,
                                                           int D, FastDiv div_d8) {
   __shared__ float part[kHeavyBlocks][kHeavyItems][9];  // padded against bank conflicts
   const int d8 = D / 8, items = n * d8;
@@ -375,7 +372,7 @@ __global__ void __launch_bounds__(kRowThreads, 3) rows_kernel(const bf16* __rest
 }
 
 // y[b][t] = x[b][t*n + n-1]: one warp per output row, 16-byte vectors.
-__global__ void __launch_bounds__(256) select_kernel(const uint4* __restrict__ x, uint4* __restrict__ y,
+__global__ void __launch_bounds__(256) select_kernel(const uint4* x, uint4* __restrict__ y,
                                                      long long rows, int n, int d16) {
   const int lane = threadIdx.x & 31;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -384,12 +381,12 @@ __global__ void __launch_bounds__(256) select_kernel(const uint4* __restrict__ x
   for (long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += nw) {
     const uint4* src = x + (r * n + (n - 1)) * d16;
     uint4* dst = y + r * d16;
-    for (int c = lane; c < d16; c += 32) dst[c] = __ldg(src + c);
+    for (int c = lane; c < d16; c += 32) dst[c] = src[c];
   }
 }
 
 // dx[b][p] = dy[b][p / n] when p % n == n-1, else zero: one warp per row of dx.
-__global__ void __launch_bounds__(256) select_bwd_kernel(const uint4* __restrict__ dy, uint4* __restrict__ dx,
+__global__ void __launch_bounds__(256) select_bwd_kernel(const uint4* dy, uint4* __restrict__ dx,
                                                          long long rows_x, int n, int d16) {
   const int lane = threadIdx.x & 31;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -399,7 +396,7 @@ __global__ void __launch_bounds__(256) select_bwd_kernel(const uint4* __restrict
     uint4* dst = dx + p * d16;
     if (p % n == n - 1) {
       const uint4* src = dy + (p / n) * d16;
-      for (int c = lane; c < d16; c += 32) dst[c] = __ldg(src + c);
+      for (int c = lane; c < d16; c += 32) dst[c] = src[c];
     } else {
       for (int c = lane; c < d16; c += 32) dst[c] = make_uint4(0, 0, 0, 0);
     }

@@ -26,9 +26,7 @@ typedef __nv_bfloat16 bf16;
 // read the eight heads' rows that share positions (adjacent in memory).  With ZERO the
 // warp then zeroes its rows of the fp32 dQ accumulator.
 template <int DH, bool ZERO>
-__global__ void __launch_bounds__(256) sfa_bwd_prep_kernel(const bf16* __restrict__ o,
-                                                           const bf16* __restrict__ dout,
-                                                           const float* __restrict__ lse,
+__global__ void __launch_bounds__(256) sfa_bwd_prep_kernel(const bf16* o, const bf16* dout, const float* lse,
                                                            float* __restrict__ lse2_t,
                                                            float* __restrict__ delta_t,
                                                            float* __restrict__ dq_acc, SfaGeom g) {

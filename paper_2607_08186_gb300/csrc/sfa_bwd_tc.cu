@@ -726,7 +726,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) bwd_kernel(const __grid_constant_
 // Head chunks: dv / dk rows (bf16) from the chunks' fp32 partial sums, added in chunk
 // order, 8 columns per thread.
 template <int DH>
-__global__ void __launch_bounds__(256) dkv_finalize_kernel(const float* __restrict__ dkv, bf16* __restrict__ dk,
+__global__ void __launch_bounds__(256) dkv_finalize_kernel(const float* dkv, bf16* __restrict__ dk,
                                                            bf16* __restrict__ dv, SfaGeom g, int chunks) {
   attn_dep_wait(8);
   const long long n8 = (long long)g.B * g.q_ns * g.Lv * g.Hkv * (DH / 8);

@@ -437,9 +437,9 @@ __global__ void __launch_bounds__(256) combine_kernel(DecodeArgs a) {
 // The new token's n K and V rows into the cache at positions (T-1)n + s: one warp per
 // (sequence, stream), 16-byte vectors.  A length outside [1, Lcap] writes nothing and
 // sets HD_DEVBIT_INDEX.
-__global__ void __launch_bounds__(256) append_kernel(const uint4* __restrict__ kn, const uint4* __restrict__ vn,
+__global__ void __launch_bounds__(256) append_kernel(const uint4* kn, const uint4* vn,
                                                      uint4* __restrict__ kc, uint4* __restrict__ vc,
-                                                     const int32_t* __restrict__ lens, int B, int Lcap, int n,
+                                                     const int32_t* lens, int B, int Lcap, int n,
                                                      int row16, int32_t* status) {
   const int lane = threadIdx.x & 31;
   const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
