@@ -773,6 +773,21 @@ __global__ void __launch_bounds__(NTHREADS, 1) decode_tc_kernel(const __grid_con
 #pragma unroll
       for (int cc = 0; cc < BN / 32; ++cc) tmem_st16(tS + cc * 16, pk + cc * 16);
       tmem_st_wait();
+      // The sequence's last tile holds cached rows past its length, which may never have been
+      // written: their P is 0, and 0 times an infinity or a NaN is NaN, so their V rows are
+      // zeroed before the PV (which waits for this thread's arrival).
+      if (base + BN > k1) {
+#pragma unroll
+        for (int u = nunits - 2; u < nunits; ++u)  // the ring's last units: this tile's V halves
+          ok = ok && __all_sync(0xffffffffu, mbar_wait(&sm.full[u % NSLOT], (u / NSLOT) & 1, abort, a.status));
+        if (!ok) break;
+        for (int r = k1 - base + row / 8; r < BN; r += 16)
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            reinterpret_cast<uint4*>(sm.ring[(nunits - 2 + (c >> 1)) % NSLOT][c & 1] + r * 64)[row % 8] =
+                make_uint4(0, 0, 0, 0);
+        fence_async_smem();
+      }
       tc_fence_before();
       mbar_arrive(&sm.p_full[i & 1]);
     }
