@@ -190,6 +190,22 @@ inline cudaError_t launch_attn(void (*kernel)(P...), long long grid, unsigned bl
   return launch_kernel(grid <= (long long)kEarlyGrid, kernel, dim3((unsigned)grid), block, smem, st, args...);
 }
 
+// dst[0, n) = src[0, n) by one warp, eight loads in flight per lane.  The loads are written
+// ahead of their stores: the compiler does not move a plain load above a store through
+// another pointer (one load in flight: the four embedding calls of 4096 tokens 164 -> 175 us,
+// an append + decoding step 30.8 -> 33.5).
+HD_DEVINLINE void warp_copy(uint4* dst, const uint4* src, int n, int lane) {
+  for (int c0 = lane; c0 < n; c0 += 256) {
+    uint4 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (c0 + 32 * k < n) v[k] = src[c0 + 32 * k];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (c0 + 32 * k < n) dst[c0 + 32 * k] = v[k];
+  }
+}
+
 HD_DEVINLINE void set_status(int32_t* st, int bit) {
   if (st) atomicOr(st, bit);
 }

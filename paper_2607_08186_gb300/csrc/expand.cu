@@ -1,7 +1,7 @@
 // Multi-stream token expansion (Eq. 1): out[b][t*n + s][:] = tables[s][ids[b][t]][:].
 //
 // HBM-bound bit copy.  One warp per output row (b, t, s): it reads the table row
-// with 16-byte loads and writes the contiguous output row with 16-byte stores, four
+// with 16-byte loads and writes the contiguous output row with 16-byte stores, eight
 // vectors in flight per lane.  Output rows are visited in memory order, so consecutive warps write
 // consecutive rows.
 #include "common.cuh"
@@ -25,16 +25,7 @@ __global__ void __launch_bounds__(256) expand_embed_kernel(const uint4* tables, 
       if (lane == 0 && s == 0) set_status(status, HD_DEVBIT_INDEX);
       continue;
     }
-    const uint4* src = tables + ((long long)s * V + id) * D16;
-    int c = lane;
-    for (; c + 96 < D16; c += 128) {
-      const uint4 a0 = src[c], a1 = src[c + 32], a2 = src[c + 64], a3 = src[c + 96];
-      dst[c] = a0;
-      dst[c + 32] = a1;
-      dst[c + 64] = a2;
-      dst[c + 96] = a3;
-    }
-    for (; c < D16; c += 32) dst[c] = src[c];
+    warp_copy(dst, tables + ((long long)s * V + id) * D16, D16, lane);
   }
 }
 

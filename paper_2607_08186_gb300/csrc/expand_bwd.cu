@@ -379,9 +379,7 @@ __global__ void __launch_bounds__(256) select_kernel(const uint4* x, uint4* __re
   grid_dep_wait();
   grid_dep_launch();
   for (long long r = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < rows; r += nw) {
-    const uint4* src = x + (r * n + (n - 1)) * d16;
-    uint4* dst = y + r * d16;
-    for (int c = lane; c < d16; c += 32) dst[c] = src[c];
+    warp_copy(y + r * d16, x + (r * n + (n - 1)) * d16, d16, lane);
   }
 }
 
@@ -395,8 +393,7 @@ __global__ void __launch_bounds__(256) select_bwd_kernel(const uint4* dy, uint4*
   for (long long p = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < rows_x; p += nw) {
     uint4* dst = dx + p * d16;
     if (p % n == n - 1) {
-      const uint4* src = dy + (p / n) * d16;
-      for (int c = lane; c < d16; c += 32) dst[c] = src[c];
+      warp_copy(dst, dy + (p / n) * d16, d16, lane);
     } else {
       for (int c = lane; c < d16; c += 32) dst[c] = make_uint4(0, 0, 0, 0);
     }

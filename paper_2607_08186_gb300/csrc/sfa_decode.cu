@@ -454,9 +454,20 @@ __global__ void __launch_bounds__(256) append_kernel(const uint4* kn, const uint
   }
   const long long dst = ((long long)b * Lcap * n + (long long)(T - 1) * n + s) * row16;
   const long long src = w * row16;
-  for (int i = lane; i < row16; i += 32) {
-    kc[dst + i] = kn[src + i];
-    vc[dst + i] = vn[src + i];
+  for (int i0 = lane; i0 < row16; i0 += 128) {  // loads ahead of the stores, as in warp_copy
+    uint4 k[4], v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (i0 + 32 * j < row16) {
+        k[j] = kn[src + i0 + 32 * j];
+        v[j] = vn[src + i0 + 32 * j];
+      }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (i0 + 32 * j < row16) {
+        kc[dst + i0 + 32 * j] = k[j];
+        vc[dst + i0 + 32 * j] = v[j];
+      }
   }
 }
 }  // namespace dec
