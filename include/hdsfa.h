@@ -168,15 +168,15 @@ hd_status_t sfa_bwd(const void* q, const void* k, const void* v, const void* o, 
                     cudaStream_t stream);
 
 /*
- * The three phases sfa_bwd runs, in order on one stream, exported so a caller
- * can overlap or time them separately.  Same sizes, mode and workspace as sfa_bwd.
+ * The backward in three phases, in order on one stream, for a caller that overlaps or
+ * times them separately or adds up dQ in fp32.  Same sizes, mode and workspace as sfa_bwd.
  *   sfa_bwd_prep     : delta = rowsum(dO * O) and lse * log2(e) into the workspace
  *                      (fp32, stream-major), and zero its fp32 dQ accumulator.
- *   sfa_bwd_main     : recompute P on visible pairs, store the finished fp32 sums of
- *                      dQ into the accumulator and write dk, dv (overwritten).
+ *   sfa_bwd_main     : recompute P on visible pairs, add every dQ contribution into
+ *                      the accumulator and write dk, dv (overwritten).
  *   sfa_bwd_finalize : dq = bf16(scale * accumulator).
  * (sfa_bwd itself runs the row terms and the main pass only: its dq is written as bf16
- * by the main pass, from the same sums.)
+ * by the main pass, from the same fp32 sums, and needs no accumulator.)
  * A later phase reads what the earlier one left in the workspace.
  * sfa_bwd_prep is itself the two halves below, for a caller that overlaps them:
  *   sfa_bwd_row_terms: the delta and lse terms only (needs o, so after sfa_fwd);
@@ -284,7 +284,7 @@ hd_status_t sfa_kv_append(const void* k_new, const void* v_new, void* k_cache, v
  *     the first call in a context also loads the library's module there, so make that
  *     first call before any stream capture.  A failed look-up returns HD_ERR_CUDA.
  *   - Sharing: every call on a device uses the same array, which keeps the last call's
- *     contents; each call clears what it reads before reading it.  Calls that may run
+ *     contents; each call writes what it reads before reading it.  Calls that may run
  *     concurrently on one device (unordered streams, several host threads) race on
  *     the array: the caller must order them.
  */

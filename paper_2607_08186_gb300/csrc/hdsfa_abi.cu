@@ -305,7 +305,7 @@ hd_status_t sfa_bwd_main(const void* q, const void* k, const void* v, const void
   BwdWs ws;
   if ((st = split_ws(g, Dh, workspace, workspace_bytes, &ws)) != HD_OK) return st;
   const float scale = resolve_scale(softmax_scale, Dh);
-  // the fp32 sums of dQ go to the workspace's accumulator (sfa_bwd takes them as bf16)
+  // the fp32 sums of dQ are added into the workspace's accumulator (sfa_bwd takes them as bf16)
   if (Dh == 256)
     return cuda_status(hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, nullptr, dk, dv, ws.lse2, ws.delta, ws.dq,
                                                         ws.dkv, g, scale, dev_status, stream));

@@ -87,7 +87,7 @@ struct Params {
   const float* lse2;   // -lse*log2(e), [B][Hq][ns][Lvp]
   const float* delta;  // -delta, the same layout
   bf16* dq;            // dQ (scaled), or null: dq_acc
-  float* dq_acc;       // unscaled fp32 dQ, when dq is null
+  float* dq_acc;       // unscaled fp32 dQ, added to what is there, when dq is null
   bf16* dk;
   bf16* dv;
   float* dkv;   // head chunks > 1: fp32 partial sums [chunks][2][B][q_ns][Lv][Hkv][DH] (dV, dK)
@@ -651,7 +651,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) bwd_kernel(const __grid_constant_
         if (f32_out) {
           float* dst;
           float m = o ? P.scale : 1.f;
-          if (kind == kDQ) {  // unscaled: sfa_bwd_finalize applies the scale
+          if (kind == kDQ) {  // unscaled (sfa_bwd_finalize applies the scale) and added: one sum per call
             dst = P.dq_acc + (((long long)it.b * G.q_nL + (long long)r * G.q_rs + it.s) * G.Hq + it.h) * DH;
           } else {
             dst = P.dkv + (2 * it.hc + o) * half + ((((long long)it.b * G.q_ns + it.s) * G.Lv + r) * G.Hkv + it.kvh) * DH;
@@ -664,10 +664,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) bwd_kernel(const __grid_constant_
             tmem_ld_wait();
             if (r < nrow) {
 #pragma unroll
-              for (int e = 0; e < 32; e += 4)
-                *reinterpret_cast<float4*>(dst + c * 32 + e) =
-                    make_float4(__uint_as_float(v[e]) * m, __uint_as_float(v[e + 1]) * m,
-                                __uint_as_float(v[e + 2]) * m, __uint_as_float(v[e + 3]) * m);
+              for (int e = 0; e < 32; e += 4) {
+                const float4 w = make_float4(__uint_as_float(v[e]) * m, __uint_as_float(v[e + 1]) * m,
+                                             __uint_as_float(v[e + 2]) * m, __uint_as_float(v[e + 3]) * m);
+                if (kind == kDQ)
+                  red_add4(dst + c * 32 + e, w.x, w.y, w.z, w.w);
+                else
+                  *reinterpret_cast<float4*>(dst + c * 32 + e) = w;
+              }
             }
           }
         } else {
@@ -817,7 +821,7 @@ static cudaError_t bwd_tc_impl(tcbwd::Params& p, long long slice, cudaStream_t s
   return launch_attn(dkv_finalize_kernel<DH>, (n8 + 255) / 256, 256, 0, st, p.dkv, p.dk, p.dv, g, p.hchunks);
 }
 
-// Dh: 64 or 128.  dq_out: bf16 dQ (scaled); null: unscaled fp32 dQ into dq_ws.  With dq_out
+// Dh: 64 or 128.  dq_out: bf16 dQ (scaled); null: unscaled fp32 dQ added into dq_ws.  With dq_out
 // the space of dq_ws is free and holds the chunks' partial sums when it is larger than dkv_ws.
 cudaError_t launch_sfa_bwd_main_tc(const void* q, const void* k, const void* v, const void* dout, void* dq_out,
                                    void* dk, void* dv, const float* lse2_ws, const float* delta_ws, float* dq_ws,

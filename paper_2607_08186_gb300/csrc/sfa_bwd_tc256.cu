@@ -93,7 +93,7 @@ struct Params {
   const float* lse2;   // -lse*log2(e), [B][Hq][ns][Lvp]
   const float* delta;  // -delta, the same layout
   bf16* dq;            // dQ (scaled), or null: dq_acc
-  float* dq_acc;       // unscaled fp32 dQ, when dq is null
+  float* dq_acc;       // unscaled fp32 dQ, added to what is there, when dq is null
   bf16* dk;
   bf16* dv;
   float* dkv;   // head chunks > 1: fp32 partial sums [chunks][2][B][q_ns][Lv][Hkv][DH] (dV, dK)
@@ -575,7 +575,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
       if (f32_out) {
         float* dst;
         float m = mul;
-        if (kind == kDQ) {  // unscaled: sfa_bwd_finalize applies the scale
+        if (kind == kDQ) {  // unscaled (sfa_bwd_finalize applies the scale) and added: one sum per call
           dst = P.dq_acc + (((long long)it.b * G.q_nL + (long long)r * G.q_rs + it.s) * G.Hq + it.head) * DH;
           m = 1.f;
         } else {
@@ -590,10 +590,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) bwd256_
           tmem_ld_wait();
           if (r < nrow) {
 #pragma unroll
-            for (int e = 0; e < 32; e += 4)
-              *reinterpret_cast<float4*>(dst + c * 32 + e) =
-                  make_float4(__uint_as_float(o[e]) * m, __uint_as_float(o[e + 1]) * m,
-                              __uint_as_float(o[e + 2]) * m, __uint_as_float(o[e + 3]) * m);
+            for (int e = 0; e < 32; e += 4) {
+              const float4 w = make_float4(__uint_as_float(o[e]) * m, __uint_as_float(o[e + 1]) * m,
+                                           __uint_as_float(o[e + 2]) * m, __uint_as_float(o[e + 3]) * m);
+              if (kind == kDQ)
+                red_add4(dst + c * 32 + e, w.x, w.y, w.z, w.w);
+              else
+                *reinterpret_cast<float4*>(dst + c * 32 + e) = w;
+            }
           }
         }
       } else {
@@ -734,7 +738,7 @@ static int head_chunks(const SfaGeom& g, long long room, long long ndq) {
 }
 }  // namespace tcbwd256
 
-// dq_out: bf16 dQ (scaled); null: unscaled fp32 dQ into dq_ws.  With dq_out the space of
+// dq_out: bf16 dQ (scaled); null: unscaled fp32 dQ added into dq_ws.  With dq_out the space of
 // dq_ws is free and holds the chunks' partial sums when it is larger than dkv_ws.
 cudaError_t launch_sfa_bwd_main_tc256(const void* q, const void* k, const void* v, const void* dout, void* dq_out,
                                       void* dk, void* dv, const float* lse2_ws, const float* delta_ws, float* dq_ws,

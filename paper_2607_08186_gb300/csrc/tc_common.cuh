@@ -146,6 +146,12 @@ HD_DEVINLINE float ex2_approx(float x) {
   return y;
 }
 
+// p[0..3] += v in memory, without reading it back (p 16-byte aligned).
+HD_DEVINLINE void red_add4(float* p, float a, float b, float c, float d) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
+               : "memory");
+}
+
 // Two fp32 -> packed bf16x2 (round to nearest even); `lo` lands in the low half.
 HD_DEVINLINE uint32_t cvt_bf16x2(float lo, float hi) {
   uint32_t r;
