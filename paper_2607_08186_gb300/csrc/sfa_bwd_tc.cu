@@ -157,7 +157,10 @@ HD_DEVINLINE Item make_item(const Params& P, int idx) {
   return it;
 }
 
-template <int DH>
+// ACC: the instantiation that adds fp32 dQ into the accumulator (sfa_bwd_main).  Its own, since
+// the reductions in the other's epilogue changed the code of its loops: 16 over 4 heads of 64,
+// 4473 positions, cross-stream 168.5 -> 173.4 us.
+template <int DH, bool ACC>
 __global__ void __launch_bounds__(NTHREADS, 1) bwd_kernel(const __grid_constant__ Params P) {
   static_assert(DH == 64 || DH == 128, "head dim 64 or 128");
   constexpr int NBUF = Smem<DH>::NBUF;
@@ -667,7 +670,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) bwd_kernel(const __grid_constant_
               for (int e = 0; e < 32; e += 4) {
                 const float4 w = make_float4(__uint_as_float(v[e]) * m, __uint_as_float(v[e + 1]) * m,
                                              __uint_as_float(v[e + 2]) * m, __uint_as_float(v[e + 3]) * m);
-                if (kind == kDQ)
+                if (ACC && kind == kDQ)
                   red_add4(dst + c * 32 + e, w.x, w.y, w.z, w.w);
                 else
                   *reinterpret_cast<float4*>(dst + c * 32 + e) = w;
@@ -812,10 +815,11 @@ static cudaError_t bwd_tc_impl(tcbwd::Params& p, long long slice, cudaStream_t s
   using namespace tcbwd;
   const SfaGeom& g = p.g;
   constexpr int smem = smem_bytes<DH>();
-  cudaError_t e = cudaFuncSetAttribute(bwd_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const auto kernel = p.dq ? bwd_kernel<DH, false> : bwd_kernel<DH, true>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const long long ndq = (long long)((g.Lq + BM - 1) / BM) * g.Hq * g.q_ns * g.B;
-  e = launch_attn(bwd_kernel<DH>, p.nkv + ndq, NTHREADS, smem, st, p);
+  e = launch_attn(kernel, p.nkv + ndq, NTHREADS, smem, st, p);
   if (e != cudaSuccess || p.hchunks == 1) return e;
   const long long n8 = slice / 8;
   return launch_attn(dkv_finalize_kernel<DH>, (n8 + 255) / 256, 256, 0, st, p.dkv, p.dk, p.dv, g, p.hchunks);
