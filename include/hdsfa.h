@@ -157,7 +157,9 @@ size_t sfa_bwd_workspace_bytes(int B, int L, int n, int Hq, int Hkv, int Dh, sfa
  *   dS = P * (dP - rowsum(dO * O)),
  *   dq = scale dS k,  dk = scale sum_{h in group} dS^T q,  dv = sum_{h in group} P^T dO.
  * Inputs q, k, v, o, dout (bf16) and lse (float32, as written by sfa_fwd).
- * Outputs dq [B][nL][Hq][Dh], dk, dv [B][nL][Hkv][Dh] (bf16, overwritten).
+ * Outputs dq [B][nL][Hq][Dh], dk, dv [B][nL][Hkv][Dh] (bf16, overwritten).  dq may lie in the
+ * buffer of an input (dout's or q's; it is then rounded from the workspace after the last
+ * read, two passes more); dk and dv may not.
  * workspace: device buffer of at least sfa_bwd_workspace_bytes(...) bytes, 256-byte
  * aligned; its contents on entry do not matter.
  */
@@ -214,7 +216,7 @@ hd_status_t sfa_bwd_finalize(void* dq, int B, int L, int n, int Hq, int Hkv, int
  *   q, o, dout, dq : bf16 [B][L][Hq][Dh]  (dense: only the final-stream rows)
  *   k, v, dk, dv   : bf16 [B][n*L][Hkv][Dh]
  *   lse            : float32 [B][Hq][L], natural log (written by sfa_fwd_final)
- * dk, dv are fully overwritten (zero for keys no final-stream query sees).
+ * dk, dv are fully overwritten (zero for keys no final-stream query sees); dq as in sfa_bwd.
  * workspace: >= sfa_bwd_final_workspace_bytes(...) bytes, 256-byte aligned.
  * Dh in {64, 128, 256}, on the same tcgen05 kernels as sfa_fwd / sfa_bwd.
  */

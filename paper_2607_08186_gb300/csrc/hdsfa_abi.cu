@@ -159,6 +159,42 @@ hd_status_t split_ws(const SfaGeom& gk, int Dh, void* ws, size_t bytes, BwdWs* o
 
 hd_status_t cuda_status(cudaError_t e) { return e == cudaSuccess ? HD_OK : HD_ERR_CUDA; }
 
+// The main pass at any head dim; dq null: fp32 dQ added into the accumulator.
+cudaError_t main_pass(const void* q, const void* k, const void* v, const void* dout, void* dq, void* dk, void* dv,
+                      const BwdWs& ws, const SfaGeom& g, int Dh, float scale, int32_t* status, cudaStream_t st) {
+  if (Dh == 256)
+    return hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, scale, status,
+                                            st);
+  return hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, Dh, scale, status,
+                                       st);
+}
+
+bool overlap(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y + b_bytes && y < x + a_bytes;
+}
+
+// The backward after its argument checks.  dQ leaves the main pass as bf16 (no accumulator to
+// clear or convert), unless dq is the buffer of an operand that the pass reads until its end
+// (dout's, say): then the sums go through the accumulator.
+cudaError_t backward(const void* q, const void* k, const void* v, const void* o, const float* lse, const void* dout,
+                     void* dq, void* dk, void* dv, const BwdWs& ws, const SfaGeom& g, int Dh, float scale,
+                     int32_t* status, cudaStream_t st) {
+  const SfaGeom gq = query_geom(g);
+  const size_t qb = (size_t)g.B * g.q_nL * g.Hq * Dh * 2, kb = (size_t)g.B * g.nL * g.Hkv * Dh * 2;
+  const bool in_place =
+      overlap(dq, qb, q, qb) || overlap(dq, qb, dout, qb) || overlap(dq, qb, k, kb) || overlap(dq, qb, v, kb);
+  cudaError_t e = hdsfa::launch_sfa_bwd_prep(o, dout, lse, ws.lse2, ws.delta, ws.dq, gq, Dh, st, in_place);
+  if (e == cudaSuccess && g.ns > g.q_ns) {
+    // a WITHIN layer's final-stream queries see only stream n-1's keys: the other rows are zero
+    e = cudaMemsetAsync(dk, 0, kb, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(dv, 0, kb, st);
+  }
+  if (e == cudaSuccess) e = main_pass(q, k, v, dout, in_place ? nullptr : dq, dk, dv, ws, g, Dh, scale, status, st);
+  if (e == cudaSuccess && in_place) e = hdsfa::launch_sfa_bwd_finalize(dq, ws.dq, gq, Dh, scale, st);
+  return e;
+}
+
 }  // namespace
 
 extern "C" {
@@ -304,13 +340,9 @@ hd_status_t sfa_bwd_main(const void* q, const void* k, const void* v, const void
   if (st != HD_OK) return st;
   BwdWs ws;
   if ((st = split_ws(g, Dh, workspace, workspace_bytes, &ws)) != HD_OK) return st;
-  const float scale = resolve_scale(softmax_scale, Dh);
-  // the fp32 sums of dQ are added into the workspace's accumulator (sfa_bwd takes them as bf16)
-  if (Dh == 256)
-    return cuda_status(hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, nullptr, dk, dv, ws.lse2, ws.delta, ws.dq,
-                                                        ws.dkv, g, scale, dev_status, stream));
-  return cuda_status(hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, nullptr, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv,
-                                                   g, Dh, scale, dev_status, stream));
+  // the fp32 sums of dQ are added into the workspace's accumulator
+  return cuda_status(main_pass(q, k, v, dout, nullptr, dk, dv, ws, g, Dh, resolve_scale(softmax_scale, Dh), dev_status,
+                               stream));
 }
 
 hd_status_t sfa_bwd_finalize(void* dq, int B, int L, int n, int Hq, int Hkv, int Dh,
@@ -341,15 +373,8 @@ hd_status_t sfa_bwd(const void* q, const void* k, const void* v, const void* o, 
   if (st != HD_OK) return st;
   BwdWs ws;
   if ((st = split_ws(g, Dh, workspace, workspace_bytes, &ws)) != HD_OK) return st;
-  // dQ leaves the main pass as bf16: no accumulator to clear or convert
-  const float scale = resolve_scale(softmax_scale, Dh);
-  cudaError_t e = hdsfa::launch_sfa_bwd_prep(o, dout, lse, ws.lse2, ws.delta, ws.dq, query_geom(g), Dh, stream, false);
-  if (e == cudaSuccess)
-    e = Dh == 256 ? hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g,
-                                                     scale, dev_status, stream)
-                  : hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, Dh,
-                                                  scale, dev_status, stream);
-  return cuda_status(e);
+  return cuda_status(backward(q, k, v, o, lse, dout, dq, dk, dv, ws, g, Dh, resolve_scale(softmax_scale, Dh), dev_status,
+                              stream));
 }
 
 // Sizes of a decode step: max_tokens bounds every sequence's length and the cache
@@ -435,24 +460,8 @@ hd_status_t sfa_bwd_final(const void* q, const void* k, const void* v, const voi
 
   BwdWs ws;
   if ((st = split_ws(g, Dh, workspace, workspace_bytes, &ws)) != HD_OK) return st;
-  const float scale = resolve_scale(softmax_scale, Dh);
-  const SfaGeom gq = query_geom(g);
-  cudaError_t e = hdsfa::launch_sfa_bwd_prep(o, dout, lse, ws.lse2, ws.delta, ws.dq, gq, Dh, stream, false);
-  if (e == cudaSuccess && mode == SFA_WITHIN) {
-    // only stream n-1's keys are seen by the final-stream queries: the other rows are zero
-    const size_t bytes = (size_t)B * n * L * Hkv * Dh * 2;
-    e = cudaMemsetAsync(dk, 0, bytes, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dv, 0, bytes, stream);
-  }
-  if (e == cudaSuccess) {
-    if (Dh == 256)
-      e = hdsfa::launch_sfa_bwd_main_tc256(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, scale,
-                                           dev_status, stream);
-    else
-      e = hdsfa::launch_sfa_bwd_main_tc(q, k, v, dout, dq, dk, dv, ws.lse2, ws.delta, ws.dq, ws.dkv, g, Dh, scale,
-                                        dev_status, stream);
-  }
-  return cuda_status(e);
+  return cuda_status(backward(q, k, v, o, lse, dout, dq, dk, dv, ws, g, Dh, resolve_scale(softmax_scale, Dh), dev_status,
+                              stream));
 }
 
 hd_status_t hd_selftest_bounded_wait(int32_t* dev_status, int32_t* dev_result, cudaStream_t stream) {
