@@ -9,9 +9,9 @@
 // module), and the entry point only looks up its address in the current context.
 //
 // The array is shared by every call on a device and keeps the previous call's
-// contents.  Nothing stale is ever read: the prep pass of each call zeroes the fp32
-// dQ accumulator and rewrites every row term (padding rows included) before the
-// main pass reads them.  Two calls that may run at the same time on one device
+// contents.  Nothing stale is ever read: every row term (padding rows included), every head
+// chunk's partial sums and, where dQ goes through the accumulator, its zeroes are written
+// earlier in the same call.  Two calls that may run at the same time on one device
 // (different streams without an ordering event, or different host threads) use the
 // same array and race; the caller orders them.
 #include "common.cuh"

@@ -7,8 +7,8 @@
 //           backward folds them in with one add / fused multiply-add.  Rows in
 //           [Lv, Lvp) get -lse2 = -inf and -delta = 0 (their P and dS vanish), from the
 //           same launch (a kernel of their own cost short layers 2 us).
-//           Also zeroes the fp32 dQ accumulator where asked to (sfa_bwd_prep; clear
-//           alone may run on another stream).
+//           Also zeroes the fp32 dQ accumulator where asked to (sfa_bwd_prep, and sfa_bwd
+//           when dq is an input's buffer; clear alone may run on another stream).
 // finalize: dq = bf16(scale * accumulator), round to nearest even.
 #include "common.cuh"
 

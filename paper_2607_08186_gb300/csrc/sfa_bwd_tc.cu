@@ -26,8 +26,9 @@
 // Measured, fwd + bwd, fused kernel (with this forward) -> this one: B=1, L=300, n=4, 32
 // over 8 heads, intra-stream 94 -> 65 us; window of 1024 at L=4096 1088 -> 1063; cross-stream
 // 2 x 4084 positions 884 -> 872; intra-stream L=4096 1753 -> 1775, 64 query heads 3487 ->
-// 3488; head dim 64, 4 x 1501 tokens, n=3 415 -> 397; the tiny configuration 31 -> 27.  Error
-// against 64 bits 3.4e-3 -> 2.4e-3 (dS is rounded once, from fp32 P).
+// 3488; head dim 64, 4 x 1501 tokens, n=3 415 -> 397; the tiny configuration 31 -> 27.  Relative
+// error of dQ and dK against 64 bits 3.4e-3 -> 2.4e-3 (dS is rounded once, from fp32 P); dV
+// 2.3e-3 as before.
 //
 // Issue order (one warp, in order, so that a region may be overwritten by the MMAs issued
 // after those that read it):
@@ -647,7 +648,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) bwd_kernel(const __grid_constant_
       tc_fence_after();
       constexpr int UPR = DH * 2 / 16, UPH = UPR / 2;  // 16-byte units per row and half row
       const int nrow = kind == kDQ ? G.Lq : G.Lv;
-      const bool f32_out = kind == kDQ ? P.dq == nullptr : P.hchunks > 1;
+      const bool f32_out = kind == kDQ ? P.dq == nullptr : P.hchunks > 1;  // (dq is null only with ACC)
 #pragma unroll 1
       for (int o = 0; o < (kind == kDQ ? 1 : 2); ++o) {  // DQ: dQ; DKV: dV, then dK
         const uint32_t to = tq + (kind == kDQ ? COL_OUT : COL_OUT + o * DH) + (DH / 2) * hc;
