@@ -193,16 +193,19 @@ inline cudaError_t launch_attn(void (*kernel)(P...), long long grid, unsigned bl
 // dst[0, n) = src[0, n) by one warp, eight loads in flight per lane.  The loads are written
 // ahead of their stores: the compiler does not move a plain load above a store through
 // another pointer (one load in flight: the four embedding calls of 4096 tokens 164 -> 175 us,
-// an append + decoding step 30.8 -> 33.5).
+// an append + decoding step 30.8 -> 33.5).  Five CTAs of 256 threads fit an SM (48 registers);
+// with four, the calls at D = 472 to 1024 took 3 % more, with four loads and six CTAs up to 10.
 HD_DEVINLINE void warp_copy(uint4* dst, const uint4* src, int n, int lane) {
-  for (int c0 = lane; c0 < n; c0 += 256) {
+  src += lane;
+  dst += lane;
+  for (int left = n - lane; left > 0; left -= 256, src += 256, dst += 256) {
     uint4 v[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-      if (c0 + 32 * k < n) v[k] = src[c0 + 32 * k];
+      if (left > 32 * k) v[k] = src[32 * k];
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-      if (c0 + 32 * k < n) dst[c0 + 32 * k] = v[k];
+      if (left > 32 * k) dst[32 * k] = v[k];
   }
 }
 

@@ -8,9 +8,9 @@
 
 namespace hdsfa {
 
-__global__ void __launch_bounds__(256) expand_embed_kernel(const uint4* tables, const int32_t* ids,
-                                                           uint4* __restrict__ out, long long rows,
-                                                           int n, int V, int D16, int32_t* status) {
+__global__ void __launch_bounds__(256, 5) expand_embed_kernel(const uint4* tables, const int32_t* ids,
+                                                              uint4* __restrict__ out, long long rows,
+                                                              int n, int V, int D16, int32_t* status) {
   const int lane = threadIdx.x & 31;
   const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;

@@ -372,8 +372,8 @@ __global__ void __launch_bounds__(kRowThreads, 3) rows_kernel(const bf16* dx, co
 }
 
 // y[b][t] = x[b][t*n + n-1]: one warp per output row, 16-byte vectors.
-__global__ void __launch_bounds__(256) select_kernel(const uint4* x, uint4* __restrict__ y,
-                                                     long long rows, int n, int d16) {
+__global__ void __launch_bounds__(256, 5) select_kernel(const uint4* x, uint4* __restrict__ y,
+                                                        long long rows, int n, int d16) {
   const int lane = threadIdx.x & 31;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
   grid_dep_wait();
@@ -384,8 +384,8 @@ __global__ void __launch_bounds__(256) select_kernel(const uint4* x, uint4* __re
 }
 
 // dx[b][p] = dy[b][p / n] when p % n == n-1, else zero: one warp per row of dx.
-__global__ void __launch_bounds__(256) select_bwd_kernel(const uint4* dy, uint4* __restrict__ dx,
-                                                         long long rows_x, int n, int d16) {
+__global__ void __launch_bounds__(256, 5) select_bwd_kernel(const uint4* dy, uint4* __restrict__ dx,
+                                                            long long rows_x, int n, int d16) {
   const int lane = threadIdx.x & 31;
   const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
   grid_dep_wait();
